@@ -17,7 +17,7 @@
 
 #include "../../include/mqo.h"
 #include "mqo_host.h"
-#include "mqo_step.cuh"
+#include "mqo_step_dense.cuh"
 
 using namespace mqo;
 
@@ -39,6 +39,9 @@ constexpr int kChunkNodes = kItemMaxNodes;  // nodes per item
 constexpr int kSplit = 512;       // row length above which the f_B kernels chunk a row
 constexpr size_t kStepSmemLimit = 110 * 1024;  // shared-memory step kernel if the graph block fits
 constexpr size_t kDiscSmemLimit = 160 * 1024;  // fused discrete kernel if the graph's bit words fit
+constexpr int kDenseMaxDegree = 1023;  // tensor-core step: neighbour counts take 10 bits
+constexpr size_t kDenseSmemLimit = 225 * 1024;  // and 32 trajectories of a member graph's x fit in shared memory
+constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3 bytes per CSR entry at most)
 constexpr int kDefaultSliceKB = 32;  // staged step kernel: gathered x rows per slice (KB)
 
 }  // namespace
@@ -60,6 +63,10 @@ struct mqo_graph_s {
   Item* d_items = nullptr;
   int32_t* d_order = nullptr;
   uint16_t* d_col16 = nullptr;  // member-local column indices (every member graph below 65536 nodes)
+  // bit matrices of dense member graphs (mqo_step_dense.cuh), built at creation
+  uint4* d_bits = nullptr;
+  int64_t* d_bits_off = nullptr;
+  int32_t max_ng = 0, max_deg = 0;
   int32_t num_items = 0;
   std::vector<int32_t> h_rp;
   std::vector<int32_t> h_off;
@@ -143,6 +150,10 @@ struct mqo_solver_s {
   bool step_ell = false;         // the current plan uses it
   const int4* ell = nullptr;     // its arrays for the current lane width
   const int2* ell_pos = nullptr;
+  // tensor-core step kernel of dense member graphs
+  bool dense_ok = false;         // the graph has bit matrices and the types allow it
+  DensePlan dense_plan{};
+  const DensePlan* dense = nullptr;  // the current plan uses it
 };
 
 namespace {
@@ -283,6 +294,44 @@ mqo_status validate(int64_t n, int64_t nnz, const int64_t* rp, const int32_t* co
   for (auto& th : pool) th.join();
   for (const Bad& b : bad)
     if (b.row >= 0) return fail(MQO_EGRAPH, "%s", b.msg);
+  return MQO_OK;
+}
+
+// Bit matrices of the member graphs (mqo_step_dense.cuh) where the step of
+// dense member graphs may use them: no weights, degrees that fit the
+// companion counts, an x block of 32 trajectories that fits in shared memory,
+// and at least kDenseFill of the matrices' cells set.
+mqo_status build_dense_bits(mqo_graph g, const std::vector<int32_t>& dmax, cudaStream_t stream) {
+  for (int32_t k = 0; k < g->G; ++k) {
+    g->max_ng = std::max(g->max_ng, g->h_off[(size_t)k + 1] - g->h_off[(size_t)k]);
+    g->max_deg = std::max(g->max_deg, dmax[(size_t)k]);
+  }
+  if (g->d_w || g->nnz == 0 || g->max_deg > kDenseMaxDegree || dense_smem_bytes(g->max_ng) > kDenseSmemLimit)
+    return MQO_OK;
+  std::vector<int64_t> off((size_t)g->G);
+  std::vector<int2> tiles;
+  int64_t vecs = 0;
+  for (int32_t k = 0; k < g->G; ++k) {
+    const int64_t nt = (g->h_off[(size_t)k + 1] - g->h_off[(size_t)k] + 127) / 128;
+    off[(size_t)k] = vecs;
+    for (int64_t t = 0; t < nt; ++t) tiles.push_back(make_int2(k, (int)t));
+    vecs += nt * nt * 128;
+  }
+  if ((double)g->nnz < kDenseFill * 128.0 * (double)vecs) return MQO_OK;
+  int2* d_tiles = nullptr;
+  mqo_status st = dalloc(&g->d_bits, (size_t)vecs, nullptr);
+  if (st == MQO_OK) st = dalloc(&g->d_bits_off, (size_t)g->G, nullptr);
+  if (st == MQO_OK) st = dalloc(&d_tiles, tiles.size(), nullptr);
+  if (st != MQO_OK) {
+    cudaFree(d_tiles);
+    return st;
+  }
+  cudaError_t e = cudaMemcpy(g->d_bits_off, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_dense_bits(g->dev(), g->d_bits_off, d_tiles, (int)tiles.size(), g->d_bits, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  cudaFree(d_tiles);
+  if (e != cudaSuccess) return fail(MQO_ECUDA, "graph bit matrices: %s", cudaGetErrorString(e));
   return MQO_OK;
 }
 
@@ -438,6 +487,7 @@ mqo_status build_graph(int32_t G, const int64_t* offs, int64_t n, int64_t nnz, c
       if (e != cudaSuccess) return cleanup(fail(MQO_ECUDA, "graph upload: %s", cudaGetErrorString(e)));
     }
   }
+  if (on_gpu && (st = build_dense_bits(g, dmax, stream)) != MQO_OK) return cleanup(st);
   *out = g;
   return MQO_OK;
 }
@@ -672,13 +722,13 @@ cudaError_t enqueue_tick(mqo_solver s) {
       for (int pass = 0; pass < 3; ++pass)
         if ((e = launch_disc(S, pass, s->work2)) != cudaSuccess) return e;
     }
-    if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos)) != cudaSuccess)
+    if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense)) != cudaSuccess)
       return e;
     if ((e = cudaEventRecord(s->ev_join, s->work2)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(s->work, s->ev_join, 0)) != cudaSuccess) return e;
     return launch_tick_end(S, s->work);
   }
-  if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos)) != cudaSuccess) return e;
+  if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense)) != cudaSuccess) return e;
   if (s->disc_smem > 0) {
     if ((e = launch_disc_graph(S, s->disc_smem, s->work)) != cudaSuccess) return e;
   } else {
@@ -767,6 +817,8 @@ mqo_status mqo_graph_destroy(mqo_graph g) {
   cudaFree(g->d_items);
   cudaFree(g->d_order);
   cudaFree(g->d_col16);
+  cudaFree(g->d_bits);
+  cudaFree(g->d_bits_off);
   cudaFree(g->d_hp);
   cudaFree(g->d_scratch);
   delete g;
@@ -908,7 +960,38 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     const bool ell_forced = ellv && strcmp(ellv, "1") == 0;
     const bool ell_off = ellv && strcmp(ellv, "0") == 0;
     if (!ellv && !force && s->ell_ok && step_wide_possible(B, p->x_dtype)) s->S.step_wide = 1;
-    if (s->step_smem > 0) use_ell(s, ell_forced || (!ell_off && !force));
+    // Dense member graphs: the tensor-core kernel, unless an environment
+    // variable above selects one of the others (MQO_STEP_KERNEL=dense: this
+    // one where possible).  Its time grows with n per row, theirs with the
+    // degree.  Measured (step of 8 to 256 graphs, B = 32 and 128, BF16): against
+    // the shared-memory kernel it wins from a mean degree of about 32 + n / 20
+    // (n = 256, degree 48: 23 us against 26; n = 800, degree 96: 29 against 34;
+    // degree 48: 45 against 41), against the staged and global ones from
+    // 16 + n / 25 (n = 800, B = 128, degree 48: 47 against 132), except where the
+    // row tiles do not fill the GPU (8 graphs of 1200 nodes, B = 32, degree 64,
+    // MaxCut: 38 against 31).
+    s->dense_ok = g->d_bits != nullptr && p->x_dtype != DT_F32 && B % kDenseGroup == 0;
+    if (s->dense_ok) {
+      s->dense_plan.bits = g->d_bits;
+      s->dense_plan.bits_off = g->d_bits_off;
+      s->dense_plan.smem = dense_smem_bytes(g->max_ng);
+      int bits = 1;
+      while ((1 << bits) <= g->max_deg) ++bits;
+      s->dense_plan.sum_bits = bits;
+      // a CTA works two row tiles at a time; a graph's tiles go to more CTAs
+      // until there are about three waves of them (2 CTAs per SM), which evens
+      // out the last wave (512 graphs of 6 tiles: 2 parts 147 us a tick, 1 part
+      // 151, 3 parts, each staging x again, 155)
+      const int pairs = (dense_tiles(g->max_ng) + 1) / 2;
+      const int ctas = g->G * (B / kDenseGroup);
+      s->dense_plan.parts = std::max(1, std::min(pairs, (6 * g->sms + ctas - 1) / ctas));
+      const double degree = (double)g->nnz / (double)g->n;
+      const bool fills = (int64_t)ctas * dense_tiles(g->max_ng) >= g->sms;
+      const double from = s->step_smem_max > 0 || !fills ? 32.0 + g->max_ng / 20.0 : 16.0 + g->max_ng / 25.0;
+      if ((!force && !ellv && !c16 && degree >= from) || (force && strcmp(force, "dense") == 0))
+        s->dense = &s->dense_plan;
+    }
+    if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
     // The fused per-graph discrete kernel runs one CTA per member graph, so
     // it is the default only with at least half as many member graphs as
     // SMs; with fewer, the node-parallel passes (several CTAs per item) fill
@@ -1050,7 +1133,7 @@ mqo_status mqo_run_timed(mqo_solver s, int64_t nticks, double* phase_ms, int64_t
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
       if (ek == cudaSuccess) ek = launch_apply(S, s->work);
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
-      if (ek == cudaSuccess) ek = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos);
+      if (ek == cudaSuccess) ek = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense);
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
       for (int pass = 0; pass < 3 && ek == cudaSuccess; ++pass) {
         if (s->disc_smem > 0) {
@@ -1104,7 +1187,7 @@ mqo_status mqo_step(mqo_solver s, int32_t nsteps) {
   const SolverDev& S = s->S;
   for (int32_t i = 0; i < nsteps; ++i) {
     CKS(cudaMemsetAsync(s->d_cnt_plain, 0, sizeof(Counters) * (size_t)S.g.num_graphs * S.B * S.R, s->work));
-    CKS(launch_step(S, s->d_cnt_plain, nullptr, nullptr, s->step_smem, s->work, s->ell, s->ell_pos));
+    CKS(launch_step(S, s->d_cnt_plain, nullptr, nullptr, s->step_smem, s->work, s->ell, s->ell_pos, s->dense));
     CKS(launch_tick_end(S, s->work));
   }
   s->host_tick += nsteps;
@@ -1203,13 +1286,19 @@ mqo_status mqo_best(mqo_solver s, int64_t* values, uint32_t* z_bits) {
   CHECK_SOLVER(s);
   const SolverDev& S = s->S;
   const size_t T = (size_t)S.g.num_graphs * S.B;
+  *s->h_pending = 0;
   {
     Scope sc(s);
+    if (s->dense) CKS(cudaMemcpyAsync(s->h_pending, S.any + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, s->work));
     if (z_bits) CKS(cudaMemcpyAsync(z_bits, S.Zbest, s->words * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s->work));
     if (values) CKS(cudaMemcpyAsync(values, S.bestv, T * sizeof(int64_t), cudaMemcpyDeviceToHost, s->work));
   }
   CKS(cudaStreamSynchronize(s->work));
   CKS(cudaStreamSynchronize(s->user));
+  if (*s->h_pending) {
+    s->poisoned = true;
+    return fail(MQO_ETIMEOUT, "a wait of the step kernel ran out");
+  }
   return MQO_OK;
 }
 
@@ -1217,17 +1306,19 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                            int32_t* replicas) {
   if (!s) return fail(MQO_EINVAL, "null solver");
   const int B = s->S.B;
-  const bool staged = s->step_smem == 0 && s->S.step_staged;
-  const int vec = s->step_smem > 0 ? 0
+  const bool staged = s->step_smem == 0 && s->S.step_staged && !s->dense;
+  const bool smem = s->step_smem > 0 || s->dense;
+  const int vec = smem ? 0
                   : (s->S.step_vec > 0 ? s->S.step_vec
                                        : (staged ? default_staged_vec(B, s->S.p.x_dtype)
                                                  : default_step_vec(B, s->S.p.x_dtype)));
   if (step_kernel)
-    *step_kernel = (s->step_smem > 0 ? 1 : 0) | (s->disc_smem > 0 ? 2 : 0) |
-                   (s->step_smem > 0 && s->S.step_wide ? 4 : 0) | (staged ? 8 : 0) | (vec << 4) |
-                   ((staged ? slice_kb(s) : 0) << 8) | ((s->step_smem > 0 && s->S.step_c16) ? (1 << 16) : 0) |
-                   ((s->step_smem > 0 && s->step_ell) ? (1 << 17) : 0);
-  if (smem_bytes) *smem_bytes = (int64_t)s->step_smem;
+    *step_kernel = (smem ? 1 : 0) | (s->disc_smem > 0 ? 2 : 0) |
+                   (s->step_smem > 0 && s->S.step_wide && !s->dense ? 4 : 0) | (staged ? 8 : 0) | (vec << 4) |
+                   ((staged ? slice_kb(s) : 0) << 8) |
+                   ((s->step_smem > 0 && s->S.step_c16 && !s->dense) ? (1 << 16) : 0) |
+                   ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0);
+  if (smem_bytes) *smem_bytes = (int64_t)(s->dense ? s->dense->smem : s->step_smem);
   if (items) *items = s->S.g.num_items;
   if (replicas) *replicas = s->S.R;
   return MQO_OK;
@@ -1267,6 +1358,14 @@ mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out) {
   CKS(cudaStreamSynchronize(s->work));
   CKS(cudaMemcpy(h.data(), s->S.st, T * sizeof(TrajState), cudaMemcpyDeviceToHost));
   CKS(cudaMemcpy(c.data(), s->S.cnt, T * R * sizeof(Counters), cudaMemcpyDeviceToHost));
+  if (s->dense) {
+    int32_t late = 0;
+    CKS(cudaMemcpy(&late, s->S.any + 3, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    if (late) {
+      s->poisoned = true;
+      return fail(MQO_ETIMEOUT, "a wait of the step kernel ran out");
+    }
+  }
   const bool mis = s->p.problem == MQO_MIS;
   for (size_t i = 0; i < T; ++i) {
     // the counters of the last tick are folded into the state by the next
@@ -1473,6 +1572,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     int slice_kb; // its slice capacity
     int c16;      // shared-memory step kernel with 16-bit column indices
     int ell;      // shared-memory step kernel with the sliced-ELL stream
+    int dense;    // tensor-core step kernel of dense member graphs
   };
   std::vector<Plan> plans;
   std::vector<size_t> steps = {0};
@@ -1485,29 +1585,31 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
       if (st > 0) {
         for (int c16 : {0, 1}) {
           if (c16 && !s->g->d_col16) continue;
-          plans.push_back({st, 0, 0, dc, 0, 0, c16, 0});
-          if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, c16, 0});
+          plans.push_back({st, 0, 0, dc, 0, 0, c16, 0, 0});
+          if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, c16, 0, 0});
         }
         if (s->ell_ok) {
-          plans.push_back({st, 0, 0, dc, 0, 0, 0, 1});
-          if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, 0, 1});
+          plans.push_back({st, 0, 0, dc, 0, 0, 0, 1, 0});
+          if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, 0, 1, 0});
         }
       } else {
         for (int v : {1, 2, 4, 8}) {
           // 16-byte lanes (8 trajectories) only for 16-bit x and momentum
           if (v == 8 && (S.p.x_dtype == DT_F32 || S.p.v_dtype == DT_F32)) continue;
-          if (B % v == 0 && B / v <= 32 && 32 % (B / v) == 0) plans.push_back({0, v, 0, dc, 0, 0, 0, 0});
+          if (B % v == 0 && B / v <= 32 && 32 % (B / v) == 0) plans.push_back({0, v, 0, dc, 0, 0, 0, 0, 0});
         }
         if (s->staged_ok)
           for (int kb : {16, 32, 64, 128}) {
             if (slice_set(s, kb).count <= 0) continue;
             for (int v : {2, 4, 8})
-              if (staged_vec_ok(B, S.p.x_dtype, v)) plans.push_back({0, v, 0, dc, 1, kb, 0, 0});
+              if (staged_vec_ok(B, S.p.x_dtype, v)) plans.push_back({0, v, 0, dc, 1, kb, 0, 0, 0});
           }
       }
     }
+  if (s->dense_ok)
+    for (size_t dc : discs) plans.push_back({steps.back(), 0, 0, dc, 0, 0, 0, 0, 1});
   const Plan keep{s->step_smem, S.step_vec, S.step_wide, s->disc_smem, S.step_staged, slice_kb(s), S.step_c16,
-                  s->step_ell ? 1 : 0};
+                  s->step_ell ? 1 : 0, s->dense ? 1 : 0};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t err = cudaEventCreate(&e0);
   if (err == cudaSuccess) err = cudaEventCreate(&e1);
@@ -1541,6 +1643,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
       S.step_c16 = pl.c16;
       if (pl.staged) use_slices(s, slice_set(s, pl.slice_kb));
       use_ell(s, pl.step_smem > 0 && pl.ell);
+      s->dense = pl.dense ? &s->dense_plan : nullptr;
       if (pl.ell && !s->step_ell) continue;  // its arrays could not be built
       if (err == cudaSuccess) err = enqueue_tick(s);  // untimed first tick
       if (err == cudaSuccess) err = cudaEventRecord(e0, s->work);
@@ -1573,6 +1676,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     S.step_c16 = pl.c16;
     if (pl.slice_kb > 0) use_slices(s, slice_set(s, pl.slice_kb));
     use_ell(s, pl.step_smem > 0 && pl.ell);
+    s->dense = pl.dense ? &s->dense_plan : nullptr;
   };
   if (err != cudaSuccess) {
     apply(keep);
@@ -1584,8 +1688,9 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
   if (s->gx16) cudaGraphExecDestroy(s->gx16);
   s->gx1 = s->gx16 = nullptr;
   if (plan_out) {
-    const bool stg = chosen.step_smem == 0 && chosen.staged;
-    *plan_out = (chosen.step_smem > 0 ? 1 : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
+    const bool stg = chosen.step_smem == 0 && chosen.staged && !chosen.dense;
+    if (chosen.dense) chosen.wide = chosen.c16 = chosen.ell = chosen.vec = 0;
+    *plan_out = (chosen.step_smem > 0 || chosen.dense ? 1 : 0) | (chosen.dense ? (1 << 18) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
                 (stg ? 8 : 0) | (chosen.vec << 4) | ((stg ? chosen.slice_kb : 0) << 8) |
                 ((chosen.step_smem > 0 && chosen.c16) ? (1 << 16) : 0) |
                 ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0);

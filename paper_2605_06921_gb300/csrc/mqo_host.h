@@ -12,14 +12,30 @@ constexpr int kPairThreads = 256;  // pair kernels: (node, trajectory) per threa
 
 enum CtrlMode : int { CTRL_MACHINE = 0, CTRL_LS_BEGIN = 1, CTRL_LS = 2, CTRL_RESET = 3 };
 
+struct DensePlan;
 // smem > 0: the shared-memory kernel with that much dynamic shared memory,
-// with the sliced-ELL neighbour stream when `ell` is given (build_ell)
+// with the sliced-ELL neighbour stream when `ell` is given (build_ell);
+// `dense`: the tensor-core kernel of dense member graphs instead
 cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, const int32_t* gflag_step,
-                        size_t smem, cudaStream_t stream, const int4* ell = nullptr, const int2* ell_pos = nullptr);
+                        size_t smem, cudaStream_t stream, const int4* ell = nullptr, const int2* ell_pos = nullptr,
+                        const DensePlan* dense = nullptr);
 // the sliced-ELL stream of the shared-memory step kernel (mqo_step_smem.cuh)
 // for `rpw` rows per warp and x rows `pitch` bytes apart, from the group
 // table `pos` (one entry per processing position)
 cudaError_t launch_ell_fill(const GraphDev& g, int rpw, int pitch, const int2* pos, int4* ell, cudaStream_t s);
+// dense member graphs on the tensor cores (mqo_step_dense.cuh): their bit
+// matrices, the CTAs per (member graph, 32 trajectories), the dynamic shared
+// memory of a CTA and the bits of the largest degree (degree < 2^sum_bits)
+struct DensePlan {
+  const uint4* bits;
+  const int64_t* bits_off;  // per member graph: first uint4
+  int32_t parts;
+  int32_t sum_bits;
+  size_t smem;
+};
+cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const int2* tiles, int num_tiles,
+                              uint4* bits, cudaStream_t s);
+size_t dense_smem_bytes(int max_ng);
 bool step_wide_possible(int B, int x_dtype);
 int default_step_vec(int B, int x_dtype);
 bool staged_vec_ok(int B, int x_dtype, int vec);

@@ -1,9 +1,11 @@
 // mqo_step.cu -- the dispatch of a tick's step to the shared-memory kernel
 // (mqo_step_smem.cuh; here with column indices from the CSR arrays, in
-// mqo_step_ell.cu with the sliced-ELL stream), the staged-gather kernel
+// mqo_step_ell.cu with the sliced-ELL stream), the tensor-core kernel of dense
+// member graphs (mqo_step_dense.cuh), the staged-gather kernel
 // (mqo_step_staged.cu) or the global-memory kernel (mqo_step_generic.cu).
 // The step itself (gradient, momentum, projection, rounding, exact
 // evaluation) is described in mqo_step.cuh.
+#include "mqo_step_dense.cuh"
 #include "mqo_step_smem.cuh"
 
 namespace mqo {
@@ -29,7 +31,7 @@ static cudaError_t launch_tv(bool wide, size_t smem, bool mis, const StepArgs& a
 }
 
 cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, const int32_t* gflag_step,
-                        size_t smem, cudaStream_t stream, const int4* ell, const int2* ell_pos) {
+                        size_t smem, cudaStream_t stream, const int4* ell, const int2* ell_pos, const DensePlan* dense) {
   StepArgs a;
   a.g = S.g;
   a.B = S.B;
@@ -57,6 +59,7 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
   a.slice_rows = S.slice_rows;
   a.slice_cols = S.slice_cols;
   const int xd = S.p.x_dtype, vd = S.p.v_dtype;
+  if (dense) return launch_step_dense(a, *dense, S.any + 3, xd, vd, stream);
   if (smem == 0 && S.step_staged) {
     // staged-gather kernel: one CTA per slice
     const int vec = S.step_vec > 0 ? S.step_vec : default_staged_vec(S.B, xd);
