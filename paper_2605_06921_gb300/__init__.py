@@ -52,7 +52,7 @@ def _plan(p):
         kern = "staged" if p & 8 else "global"
     return {"step_kernel": kern, "discrete_kernel": "graph" if p & 2 else "pairs", "lanes_vec": (p >> 4) & 15,
             "slice_kb": (p >> 8) & 255, "col16": bool(p & (1 << 16)), "ell": bool(p & (1 << 17)),
-            "dense": bool(p & (1 << 18))}
+            "dense": bool(p & (1 << 18)), "small": bool(p & (1 << 19))}
 
 
 class TrajInfo(C.Structure):

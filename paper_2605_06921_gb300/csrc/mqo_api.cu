@@ -39,6 +39,8 @@ constexpr int kChunkNodes = kItemMaxNodes;  // nodes per item
 constexpr int kSplit = 512;       // row length above which the f_B kernels chunk a row
 constexpr size_t kStepSmemLimit = 110 * 1024;  // shared-memory step kernel if the graph block fits
 constexpr size_t kDiscSmemLimit = 160 * 1024;  // fused discrete kernel if the graph's bit words fit
+constexpr size_t kSmallSmemLimit = 200 * 1024;  // multi-tick kernel: a member graph and its trajectories fit
+constexpr int kSmallTicks = 4096;               // ticks per launch of that kernel
 constexpr int kDenseMaxDegree = 1023;  // tensor-core step: neighbour counts take 10 bits
 constexpr size_t kDenseSmemLimit = 225 * 1024;  // and 32 trajectories of a member graph's x fit in shared memory
 constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3 bytes per CSR entry at most)
@@ -154,6 +156,10 @@ struct mqo_solver_s {
   bool dense_ok = false;         // the graph has bit matrices and the types allow it
   DensePlan dense_plan{};
   const DensePlan* dense = nullptr;  // the current plan uses it
+  // many ticks of small member graphs in one launch (mqo_small.cu)
+  size_t small_smem = 0;  // > 0: possible, with this much dynamic shared memory
+  int small_threads = 0;
+  bool small = false;     // the current plan uses it
 };
 
 namespace {
@@ -987,9 +993,48 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
       s->dense_plan.parts = std::max(1, std::min(pairs, (6 * g->sms + ctas - 1) / ctas));
       const double degree = (double)g->nnz / (double)g->n;
       const bool fills = (int64_t)ctas * dense_tiles(g->max_ng) >= g->sms;
-      const double from = s->step_smem_max > 0 || !fills ? 32.0 + g->max_ng / 20.0 : 16.0 + g->max_ng / 25.0;
-      if ((!force && !ellv && !c16 && degree >= from) || (force && strcmp(force, "dense") == 0))
+      // MaxCut meets x inside the box for longer (rows summed in CSR order), and
+      // 11-bit significands leave fewer sums exact: a higher line against the
+      // shared-memory kernel, and none for float16 (407 graphs, n = 164, degree
+      // 46, B = 128: 164 us a tick against 142)
+      const bool cut = p->problem == PROB_MAXCUT;
+      const double from = s->step_smem_max > 0 || !fills ? (cut ? 48.0 + g->max_ng / 16.0 : 32.0 + g->max_ng / 20.0)
+                                                         : 16.0 + g->max_ng / 25.0;
+      const bool few_exact = cut && p->x_dtype == DT_F16 && s->step_smem_max > 0;
+      if ((!force && !ellv && !c16 && degree >= from && !few_exact) || (force && strcmp(force, "dense") == 0))
         s->dense = &s->dense_plan;
+    }
+    // Small member graphs: the multi-tick kernel, unless an environment
+    // variable selects one of the tick's kernels (MQO_TICK_KERNEL=ticks: never,
+    // small: wherever it is possible).
+    {
+      int64_t work = 0;
+      int pairs = 0;
+      size_t smem = 0;
+      for (int32_t k = 0; k < g->G; ++k) {
+        const int32_t ng = g->h_off[k + 1] - g->h_off[k];
+        const int32_t nz = g->h_rp[(size_t)g->h_off[k + 1]] - g->h_rp[(size_t)g->h_off[k]];
+        work = std::max(work, (int64_t)nz * B);
+        pairs = (int)std::max<int64_t>(pairs, std::min<int64_t>((int64_t)ng * B, 1 << 20));
+        if (ng >= 65536 || (int64_t)ng * B > (1 << 20)) smem = SIZE_MAX;
+        else smem = std::max(smem, small_smem_bytes(B, p->x_dtype, p->v_dtype, ng, nz, g->d_w != nullptr));
+      }
+      if (p->pool_k == 0 && S.R == 1 && smem <= kSmallSmemLimit) {
+        s->small_smem = smem;
+        s->small_threads = std::min(1024, std::max(128, (pairs + 127) / 128 * 128));
+        const char* tk = getenv("MQO_TICK_KERNEL");
+        const bool other = force || ellv || c16 || getenv("MQO_DISC_KERNEL") || getenv("MQO_SERIAL_TICK");
+        // Its tick takes about 0.8 us, 0.8 ns per (node, trajectory) pair and
+        // 0.06 ns per (entry, trajectory) pair of the largest member graph, and
+        // there is one CTA per SM; a tick of the kernels takes 11 us and up
+        // (n = 200, B = 1: 1.0 against 11.7; n = 400, degree 24, B = 8: 8.3 against
+        // 12.8; n = 200, degree 24, B = 32: 12.9 against 19.5, 300 graphs 26
+        // against 28; n = 400, degree 24, B = 32: 25 against 21).
+        const double us = 0.8 + 0.8e-3 * pairs + 0.06e-3 * (double)work;
+        const int waves = (g->G + g->sms - 1) / g->sms;
+        const bool faster = us <= 11.0 && us * waves <= 22.0;
+        s->small = tk ? strcmp(tk, "small") == 0 : !other && faster;
+      }
     }
     if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
     // The fused per-graph discrete kernel runs one CTA per member graph, so
@@ -1069,22 +1114,13 @@ mqo_status mqo_init(mqo_solver s) {
   CHECK_SOLVER(s);
   Scope sc(s);
   SolverDev& S = s->S;
-  CKS(cudaMemsetAsync(S.V, 0, s->v_bytes, s->work));
-  for (uint32_t* w : {S.ZX0, S.ZX1, S.Zbest, S.Zwork, S.Zaux, S.Zfree, S.Zdrop})
-    CKS(cudaMemsetAsync(w, 0, s->words * sizeof(uint32_t), s->work));
-  CKS(cudaMemsetAsync(S.owner, 0x7f, s->pairs * sizeof(int32_t), s->work));
-  CKS(cudaMemsetAsync(S.pa, 0xff, s->pairs * sizeof(int32_t), s->work));
-  CKS(cudaMemsetAsync(S.pb, 0xff, s->pairs * sizeof(int32_t), s->work));
-  CKS(cudaMemsetAsync(S.gain, 0, s->pairs * sizeof(int32_t), s->work));
-  CKS(cudaMemsetAsync(s->d_cnt_plain, 0, sizeof(Counters) * (size_t)S.g.num_graphs * S.B * S.R, s->work));
   if (S.K > 0) {
     CKS(cudaMemsetAsync(S.Pool, 0, (size_t)S.g.n * S.Kw * sizeof(uint32_t), s->work));
     CKS(cudaMemsetAsync(S.pval, 0, (size_t)S.g.num_graphs * S.K * sizeof(int64_t), s->work));
     CKS(cudaMemsetAsync(S.psrc, 0, (size_t)S.g.num_graphs * S.K * sizeof(int32_t), s->work));
     CKS(cudaMemsetAsync(S.pbase, 0xff, (size_t)S.g.num_graphs * S.B * sizeof(int32_t), s->work));
   }
-  CKS(launch_state_init(S, s->work));
-  CKS(launch_apply(S, s->work));
+  CKS(launch_init(S, s->d_cnt_plain, s->work));
   return MQO_OK;
 }
 
@@ -1092,6 +1128,12 @@ mqo_status mqo_run(mqo_solver s, int64_t nticks) {
   CHECK_SOLVER(s);
   if (nticks < 0) return fail(MQO_EINVAL, "nticks < 0");
   Scope sc(s);
+  if (s->small) {
+    for (int64_t left = nticks; left > 0; left -= kSmallTicks)
+      CKS(launch_small(s->S, (int)std::min<int64_t>(left, kSmallTicks), nullptr, s->small_threads, s->small_smem, s->work));
+    s->host_tick += nticks;
+    return MQO_OK;
+  }
   if (!s->gx1) {
     CKS(capture(s, 1, &s->gx1));
     CKS(capture(s, 16, &s->gx16));
@@ -1185,6 +1227,12 @@ mqo_status mqo_step(mqo_solver s, int32_t nsteps) {
   if (nsteps < 0) return fail(MQO_EINVAL, "nsteps < 0");
   Scope sc(s);
   const SolverDev& S = s->S;
+  if (s->small) {
+    for (int32_t left = nsteps; left > 0; left -= kSmallTicks)
+      CKS(launch_small(S, std::min(left, kSmallTicks), s->d_cnt_plain, s->small_threads, s->small_smem, s->work));
+    s->host_tick += nsteps;
+    return MQO_OK;
+  }
   for (int32_t i = 0; i < nsteps; ++i) {
     CKS(cudaMemsetAsync(s->d_cnt_plain, 0, sizeof(Counters) * (size_t)S.g.num_graphs * S.B * S.R, s->work));
     CKS(launch_step(S, s->d_cnt_plain, nullptr, nullptr, s->step_smem, s->work, s->ell, s->ell_pos, s->dense));
@@ -1317,7 +1365,8 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                    (s->step_smem > 0 && s->S.step_wide && !s->dense ? 4 : 0) | (staged ? 8 : 0) | (vec << 4) |
                    ((staged ? slice_kb(s) : 0) << 8) |
                    ((s->step_smem > 0 && s->S.step_c16 && !s->dense) ? (1 << 16) : 0) |
-                   ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0);
+                   ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0) |
+                   (s->small ? (1 << 19) : 0);
   if (smem_bytes) *smem_bytes = (int64_t)(s->dense ? s->dense->smem : s->step_smem);
   if (items) *items = s->S.g.num_items;
   if (replicas) *replicas = s->S.R;
@@ -1573,6 +1622,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     int c16;      // shared-memory step kernel with 16-bit column indices
     int ell;      // shared-memory step kernel with the sliced-ELL stream
     int dense;    // tensor-core step kernel of dense member graphs
+    int small;    // the multi-tick kernel runs the ticks
   };
   std::vector<Plan> plans;
   std::vector<size_t> steps = {0};
@@ -1608,8 +1658,14 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     }
   if (s->dense_ok)
     for (size_t dc : discs) plans.push_back({steps.back(), 0, 0, dc, 0, 0, 0, 0, 1});
+  for (Plan& pl : plans) pl.small = 0;
   const Plan keep{s->step_smem, S.step_vec, S.step_wide, s->disc_smem, S.step_staged, slice_kb(s), S.step_c16,
-                  s->step_ell ? 1 : 0, s->dense ? 1 : 0};
+                  s->step_ell ? 1 : 0, s->dense ? 1 : 0, s->small ? 1 : 0};
+  if (s->small_smem > 0 && !s->small) {
+    Plan pl = keep;
+    pl.small = 1;
+    plans.push_back(pl);
+  }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t err = cudaEventCreate(&e0);
   if (err == cudaSuccess) err = cudaEventCreate(&e1);
@@ -1645,9 +1701,15 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
       use_ell(s, pl.step_smem > 0 && pl.ell);
       s->dense = pl.dense ? &s->dense_plan : nullptr;
       if (pl.ell && !s->step_ell) continue;  // its arrays could not be built
-      if (err == cudaSuccess) err = enqueue_tick(s);  // untimed first tick
+      auto run = [&](int32_t n) {
+        if (pl.small) return launch_small(S, n, nullptr, s->small_threads, s->small_smem, s->work);
+        cudaError_t e = cudaSuccess;
+        for (int32_t k = 0; k < n && e == cudaSuccess; ++k) e = enqueue_tick(s);
+        return e;
+      };
+      if (err == cudaSuccess) err = run(1);  // untimed first tick
       if (err == cudaSuccess) err = cudaEventRecord(e0, s->work);
-      for (int32_t k = 0; k < ticks && err == cudaSuccess; ++k) err = enqueue_tick(s);
+      if (err == cudaSuccess) err = run(ticks);
       if (err == cudaSuccess) err = cudaEventRecord(e1, s->work);
       if (err == cudaSuccess) err = cudaEventSynchronize(e1);
       float ms = 0.0f;
@@ -1677,6 +1739,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     if (pl.slice_kb > 0) use_slices(s, slice_set(s, pl.slice_kb));
     use_ell(s, pl.step_smem > 0 && pl.ell);
     s->dense = pl.dense ? &s->dense_plan : nullptr;
+    s->small = pl.small != 0;
   };
   if (err != cudaSuccess) {
     apply(keep);
@@ -1690,7 +1753,8 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
   if (plan_out) {
     const bool stg = chosen.step_smem == 0 && chosen.staged && !chosen.dense;
     if (chosen.dense) chosen.wide = chosen.c16 = chosen.ell = chosen.vec = 0;
-    *plan_out = (chosen.step_smem > 0 || chosen.dense ? 1 : 0) | (chosen.dense ? (1 << 18) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
+    *plan_out = (chosen.step_smem > 0 || chosen.dense ? 1 : 0) | (chosen.dense ? (1 << 18) : 0) |
+                (chosen.small ? (1 << 19) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
                 (stg ? 8 : 0) | (chosen.vec << 4) | ((stg ? chosen.slice_kb : 0) << 8) |
                 ((chosen.step_smem > 0 && chosen.c16) ? (1 << 16) : 0) |
                 ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0);

@@ -42,6 +42,11 @@ bool staged_vec_ok(int B, int x_dtype, int vec);
 int default_staged_vec(int B, int x_dtype);
 size_t step_smem_bytes(int B, int x_dtype, int problem, int max_ng);
 
+// small member graphs: `count` ticks (plain == nullptr) or plain steps in one
+// launch, advancing the tick number (mqo_small.cu)
+size_t small_smem_bytes(int B, int x_dtype, int v_dtype, int ng, int nnz, bool weighted);
+cudaError_t launch_small(const SolverDev& S, int count, Counters* plain, int threads, size_t smem, cudaStream_t s);
+
 cudaError_t launch_ctrl(const SolverDev& S, int mode, const uint8_t* mask, cudaStream_t stream);
 cudaError_t launch_apply(const SolverDev& S, cudaStream_t stream);
 cudaError_t launch_disc(const SolverDev& S, int pass, cudaStream_t stream);
@@ -54,7 +59,7 @@ cudaError_t launch_counters_out(const SolverDev& S, const Counters* c, int64_t* 
                                 int kind, cudaStream_t stream);
 cudaError_t launch_objective(const SolverDev& S, double* out, cudaStream_t stream);
 cudaError_t launch_ls_merge(const SolverDev& S, const TrajState* saved, cudaStream_t stream);
-cudaError_t launch_state_init(const SolverDev& S, cudaStream_t stream);
+cudaError_t launch_init(const SolverDev& S, Counters* plain, cudaStream_t stream);
 cudaError_t launch_any_pending(const SolverDev& S, int32_t* out, cudaStream_t stream);
 // device check of the CSR entries (range, no self loop, strictly ascending
 // rows, weights in {-1,+1}, no edge between member graphs, a reverse entry
