@@ -120,6 +120,8 @@ struct mqo_solver_s {
   size_t disc_smem = 0;  // > 0: fused per-graph discrete kernel with this much dynamic smem
   size_t step_smem_max = 0;  // smem the shared-memory step kernel needs (0: not possible)
   size_t disc_smem_max = 0;  // smem the fused discrete kernel needs (0: not possible)
+  size_t disc_bits_max = 0;  // smem of its form on bit matrices (0: not possible)
+  bool disc_bits = false;    // the current plan uses that form (disc_smem bytes)
   int64_t host_tick = 0;
   Counters* d_cnt_plain = nullptr;
   Counters* d_eval = nullptr;
@@ -704,6 +706,12 @@ bool serial_tick() {
   return e && strcmp(e, "1") == 0;
 }
 
+// the discrete passes fused into one launch
+cudaError_t launch_disc_fused(mqo_solver s, cudaStream_t stream) {
+  if (s->disc_bits) return launch_disc_bits(s->S, s->g->d_bits, s->g->d_bits_off, s->disc_smem, stream);
+  return launch_disc_graph(s->S, s->disc_smem, stream);
+}
+
 cudaError_t enqueue_tick(mqo_solver s) {
   cudaError_t e;
   const SolverDev& S = s->S;
@@ -723,7 +731,7 @@ cudaError_t enqueue_tick(mqo_solver s) {
     if ((e = cudaEventRecord(s->ev_fork, s->work)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(s->work2, s->ev_fork, 0)) != cudaSuccess) return e;
     if (s->disc_smem > 0) {
-      if ((e = launch_disc_graph(S, s->disc_smem, s->work2)) != cudaSuccess) return e;
+      if ((e = launch_disc_fused(s, s->work2)) != cudaSuccess) return e;
     } else {
       for (int pass = 0; pass < 3; ++pass)
         if ((e = launch_disc(S, pass, s->work2)) != cudaSuccess) return e;
@@ -736,7 +744,7 @@ cudaError_t enqueue_tick(mqo_solver s) {
   }
   if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense)) != cudaSuccess) return e;
   if (s->disc_smem > 0) {
-    if ((e = launch_disc_graph(S, s->disc_smem, s->work)) != cudaSuccess) return e;
+    if ((e = launch_disc_fused(s, s->work)) != cudaSuccess) return e;
   } else {
     for (int pass = 0; pass < 3; ++pass)
       if ((e = launch_disc(S, pass, s->work)) != cudaSuccess) return e;
@@ -750,7 +758,7 @@ cudaError_t enqueue_ls_tick(mqo_solver s, int mode) {
   if ((e = launch_ctrl(S, mode, nullptr, s->work)) != cudaSuccess) return e;
   if ((e = launch_apply(S, s->work)) != cudaSuccess) return e;
   if (s->disc_smem > 0) {
-    if ((e = launch_disc_graph(S, s->disc_smem, s->work)) != cudaSuccess) return e;
+    if ((e = launch_disc_fused(s, s->work)) != cudaSuccess) return e;
   } else {
     for (int pass = 0; pass < 3; ++pass)
       if ((e = launch_disc(S, pass, s->work)) != cudaSuccess) return e;
@@ -1048,6 +1056,13 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     const bool few = 2 * g->G < g->sms;
     s->disc_smem_max = (B >= 32 && dneed <= kDiscSmemLimit && (!few || fused)) ? dneed : 0;
     s->disc_smem = pairs ? 0 : s->disc_smem_max;
+    // Member graphs with bit matrices: the form that follows the trajectories in
+    // a round (MQO_DISC_KERNEL=bits where possible; the others exclude it).
+    s->disc_bits_max = g->d_bits != nullptr && B >= 32 ? disc_bits_smem_bytes(p->problem, max_ng) : 0;
+    if (s->disc_bits_max > 0 && (!dforce || strcmp(dforce, "bits") == 0)) {
+      s->disc_bits = true;
+      s->disc_smem = s->disc_bits_max;
+    }
   }
   const size_t TR = (size_t)T * S.R;
   S.K = p->pool_k;
@@ -1179,7 +1194,7 @@ mqo_status mqo_run_timed(mqo_solver s, int64_t nticks, double* phase_ms, int64_t
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
       for (int pass = 0; pass < 3 && ek == cudaSuccess; ++pass) {
         if (s->disc_smem > 0) {
-          if (pass == 0) ek = launch_disc_graph(S, s->disc_smem, s->work);  // all three passes fused
+          if (pass == 0) ek = launch_disc_fused(s, s->work);  // all three passes fused
         } else {
           ek = launch_disc(S, pass, s->work);
         }
@@ -1623,6 +1638,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     int ell;      // shared-memory step kernel with the sliced-ELL stream
     int dense;    // tensor-core step kernel of dense member graphs
     int small;    // the multi-tick kernel runs the ticks
+    int dbits;    // fused discrete passes on bit matrices
   };
   std::vector<Plan> plans;
   std::vector<size_t> steps = {0};
@@ -1658,9 +1674,20 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     }
   if (s->dense_ok)
     for (size_t dc : discs) plans.push_back({steps.back(), 0, 0, dc, 0, 0, 0, 0, 1});
-  for (Plan& pl : plans) pl.small = 0;
+  for (Plan& pl : plans) pl.small = pl.dbits = 0;
+  if (s->disc_bits_max > 0) {
+    // every step plan also with the discrete passes on bit matrices
+    const size_t count = plans.size();
+    for (size_t i = 0; i < count; ++i)
+      if (plans[i].disc_smem == 0) {
+        Plan pl = plans[i];
+        pl.disc_smem = s->disc_bits_max;
+        pl.dbits = 1;
+        plans.push_back(pl);
+      }
+  }
   const Plan keep{s->step_smem, S.step_vec, S.step_wide, s->disc_smem, S.step_staged, slice_kb(s), S.step_c16,
-                  s->step_ell ? 1 : 0, s->dense ? 1 : 0, s->small ? 1 : 0};
+                  s->step_ell ? 1 : 0, s->dense ? 1 : 0, s->small ? 1 : 0, s->disc_bits ? 1 : 0};
   if (s->small_smem > 0 && !s->small) {
     Plan pl = keep;
     pl.small = 1;
@@ -1695,6 +1722,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
       S.step_vec = pl.vec;
       S.step_wide = pl.wide;
       s->disc_smem = pl.disc_smem;
+      s->disc_bits = pl.dbits != 0;
       S.step_staged = pl.staged;
       S.step_c16 = pl.c16;
       if (pl.staged) use_slices(s, slice_set(s, pl.slice_kb));
@@ -1734,6 +1762,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     S.step_vec = pl.vec;
     S.step_wide = pl.wide;
     s->disc_smem = pl.disc_smem;
+    s->disc_bits = pl.dbits != 0;
     S.step_staged = pl.staged;
     S.step_c16 = pl.c16;
     if (pl.slice_kb > 0) use_slices(s, slice_set(s, pl.slice_kb));
