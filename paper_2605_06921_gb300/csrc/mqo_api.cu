@@ -1288,7 +1288,10 @@ mqo_status mqo_evaluate(mqo_solver s, const uint32_t* z_bits, int64_t* value, in
   Scope sc(s);
   const SolverDev& S = s->S;
   CKS(cudaMemsetAsync(s->d_eval, 0, sizeof(Counters) * (size_t)S.g.num_graphs * S.B * S.R, s->work));
-  CKS(launch_eval(S, z_bits, s->d_eval, s->work));
+  if (s->g->d_bits && S.B >= 32)
+    CKS(launch_eval_bits(S, s->g->d_bits, s->g->d_bits_off, s->g->max_ng, z_bits, s->d_eval, s->work));
+  else
+    CKS(launch_eval(S, z_bits, s->d_eval, s->work));
   CKS(launch_counters_out(S, s->d_eval, value, conflicts, uncovered, 1, s->work));
   return MQO_OK;
 }

@@ -396,6 +396,97 @@ __global__ void __launch_bounds__(kDbThreads) k_disc_bits(SolverDev S, const uin
   }
 }
 
+// Exact evaluation of given bits (k_eval, mqo_tick.cu) for member graphs with
+// bit matrices: one CTA per (member graph, word of 32 trajectories, part of the
+// rows); the sets as bit vectors in shared memory, a thread per row, counts by
+// popc (64 graphs of 750 nodes, degree 112: 204 us with a load per neighbour and
+// trajectory, 36 us now).
+__global__ void __launch_bounds__(256) k_eval_bits(SolverDev S, const uint4* __restrict__ bits,
+                                                   const int64_t* __restrict__ bits_off, int parts,
+                                                   const uint32_t* __restrict__ z, Counters* out) {
+  __shared__ __align__(16) uint32_t s_z[32][kDbWords];
+  __shared__ int s_cnt[32][3];
+  const int part = blockIdx.x % parts;
+  const int wk = (blockIdx.x / parts) % S.Bw, g = blockIdx.x / parts / S.Bw;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool mis = S.p.problem == PROB_MIS;
+  const int32_t off = S.g.node_off[g];
+  const int n = S.g.node_off[g + 1] - off;
+  const int tiles = (n + 255) / 256;
+  if (part >= tiles) return;
+  const BitRows rows{reinterpret_cast<const uint32_t*>(bits + bits_off[g]), (n + 127) >> 7};
+  if (threadIdx.x < 96) s_cnt[threadIdx.x / 3][threadIdx.x % 3] = 0;
+  for (int w = warp; w < 4 * rows.nc; w += 8) {
+    const int v = 32 * w + unperm(lane);
+    uint32_t x = v < n ? z[(int64_t)(off + v) * S.Bw + wk] : 0u;
+    for (int b = 0; b < 32; ++b) {
+      const unsigned m = __ballot_sync(0xffffffffu, (x >> b) & 1u);
+      if (lane == b) s_z[b][w] = m;
+    }
+  }
+  __syncthreads();
+  for (int tile = part; tile < tiles; tile += parts) {
+    const int v = tile * 256 + threadIdx.x;
+    const bool in = v < n;
+    const uint32_t own = in ? z[(int64_t)(off + v) * S.Bw + wk] : 0u;
+    int deg = 0;
+    // eight trajectories at a time, so that their counts stay in registers
+    for (int b0 = 0; b0 < 32; b0 += 8) {
+      int cnt[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) cnt[k] = 0;
+      for (int c = 0; in && c < rows.nc; ++c) {
+        const uint4 r = rows.piece(v, c);
+        if (b0 == 0) deg += __popc(r.x) + __popc(r.y) + __popc(r.z) + __popc(r.w);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint4 m = *reinterpret_cast<const uint4*>(&s_z[b0 + k][4 * c]);
+          cnt[k] += __popc(r.x & m.x) + __popc(r.y & m.y) + __popc(r.z & m.z) + __popc(r.w & m.w);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const bool zv = (own >> (b0 + k)) & 1u;
+        int a0, a1, a2;
+        if (mis) {
+          a0 = zv;
+          a1 = zv ? cnt[k] : 0;
+          a2 = !zv && cnt[k] == 0;
+        } else {
+          const int as = 2 * cnt[k] - deg;
+          a0 = zv ? deg - cnt[k] : cnt[k];
+          a1 = !(zv ? as <= -1 : as >= 0);
+          a2 = (zv ? as : -as) > 0;
+        }
+        a0 = __reduce_add_sync(0xffffffffu, in ? a0 : 0);
+        a1 = __reduce_add_sync(0xffffffffu, in ? a1 : 0);
+        a2 = __reduce_add_sync(0xffffffffu, in ? a2 : 0);
+        if (lane == 0) {
+          if (a0) atomicAdd(&s_cnt[b0 + k][0], a0);
+          if (a1) atomicAdd(&s_cnt[b0 + k][1], a1);
+          if (a2) atomicAdd(&s_cnt[b0 + k][2], a2);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 96) {
+    const int b = threadIdx.x / 3, k = threadIdx.x % 3;
+    const int val = s_cnt[b][k];
+    if (val) {
+      Counters* c = out + ((int64_t)g * S.B + wk * 32 + b) * S.R;
+      atomicAdd(k == 0 ? &c->value : k == 1 ? &c->a : &c->b, (unsigned long long)val);
+    }
+  }
+}
+
+cudaError_t launch_eval_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, int max_ng,
+                             const uint32_t* z, Counters* out, cudaStream_t stream) {
+  const int parts = (max_ng + 255) / 256;
+  k_eval_bits<<<S.g.num_graphs * S.Bw * parts, 256, 0, stream>>>(S, bits, bits_off, parts, z, out);
+  return cudaGetLastError();
+}
+
 size_t disc_bits_smem_bytes(int problem, int max_ng) {
   const size_t n = (size_t)max_ng;
   return n * (3 * 4 + kDbBatch * (4 + 4 + 2 + (problem == PROB_MIS ? 0 : 4))) + 16;

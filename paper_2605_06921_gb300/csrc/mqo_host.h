@@ -59,6 +59,8 @@ cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_
 cudaError_t launch_tick_end(const SolverDev& S, cudaStream_t stream);
 cudaError_t launch_round_bits(const SolverDev& S, uint32_t* z, cudaStream_t stream);
 cudaError_t launch_eval(const SolverDev& S, const uint32_t* z, Counters* out, cudaStream_t stream);
+cudaError_t launch_eval_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, int max_ng,
+                             const uint32_t* z, Counters* out, cudaStream_t stream);
 cudaError_t launch_counters_out(const SolverDev& S, const Counters* c, int64_t* value, int64_t* a, int64_t* b,
                                 int kind, cudaStream_t stream);
 cudaError_t launch_objective(const SolverDev& S, double* out, cudaStream_t stream);

@@ -16,6 +16,8 @@
 // share one bit word of a node (G = min(B,32) lanes) form a group; MIS set
 // logic is done on whole words: the group splits v's neighbour list, ORs
 // (or once/twice-accumulates) the neighbours' words and reduces by shuffles.
+#include <algorithm>
+
 #include "mqo_machine.cuh"
 
 namespace mqo {
@@ -311,17 +313,37 @@ cudaError_t launch_round_bits(const SolverDev& S, uint32_t* z, cudaStream_t stre
   return cudaGetLastError();
 }
 
+// The readout kernels sum a pair's neighbours kAhead at a time, so that many
+// loads are in flight, and split the items until every SM has about eight
+// CTAs (64 graphs of 750 nodes, 32 trajectories: objective, evaluation and
+// rounding together 430 us -> 144 us; one neighbour at a time and a CTA per item
+// they waited for one L2 load after the other).
+constexpr int kAhead = 8;
+static SolverDev split_items(const SolverDev& S, int sms) {
+  SolverDev D = S;
+  const int target = 8 * sms;
+  D.split = S.g.num_items >= target ? 1 : std::min(16, (target + S.g.num_items - 1) / S.g.num_items);
+  return D;
+}
+static int sm_count() {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 // exact evaluation of given bits: MIS (size, conflicting edges x2, uncovered);
 // MaxCut (2*cut, non-fixed, positive gain)
-__global__ void __launch_bounds__(kPairThreads) k_eval(SolverDev S, const uint32_t* z, Counters* out) {
+__global__ void __launch_bounds__(kPairThreads) k_eval(SolverDev S, const uint32_t* __restrict__ z, Counters* out) {
   __shared__ unsigned long long s_cnt[4 * 128];
   const int B = S.B, Bw = S.Bw;
   const bool mis = S.p.problem == PROB_MIS;
-  const int32_t* rp = S.g.row_ptr;
-  const int32_t* col = S.g.col;
-  const int8_t* wts = S.g.w;
-  const int it = blockIdx.x;
-  const Item item = S.g.items[it];
+  const int32_t* __restrict__ rp = S.g.row_ptr;
+  const int32_t* __restrict__ col = S.g.col;
+  const int8_t* __restrict__ wts = S.g.w;
+  int it;
+  Item item;
+  if (!item_slice(S, it, item)) return;
   for (int i = threadIdx.x; i < 4 * B; i += blockDim.x) s_cnt[i] = 0ull;
   __syncthreads();
   long long a0 = 0, a1 = 0, a2 = 0;
@@ -331,19 +353,31 @@ __global__ void __launch_bounds__(kPairThreads) k_eval(SolverDev S, const uint32
     const int64_t v = c.v;
     const int b = c.b;
     const bool zv = get_bit(z, v, Bw, b);
-    if (mis) {
-      int cnt = 0;
-      for (int32_t j = rp[v]; j < rp[v + 1]; ++j) cnt += get_bit(z, col[j], Bw, b);
-      a0 += zv;
-      a1 += zv ? cnt : 0;
-      a2 += !zv && cnt == 0;
-    } else {
-      int P = 0, W = 0;
-      for (int32_t j = rp[v]; j < rp[v + 1]; ++j) {
-        const int w = wts ? (int)wts[j] : 1;
-        W += w;
-        if (get_bit(z, col[j], Bw, b)) P += w;
+    // neighbours (their weights) in the set, and all of them
+    const int32_t j1 = rp[v + 1];
+    int32_t j = rp[v];
+    int P = 0, W = wts ? 0 : j1 - j;
+    for (; j + kAhead <= j1; j += kAhead) {
+      bool in[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) in[k] = get_bit(z, col[j + k], Bw, b);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int w = wts ? (int)wts[j + k] : 1;
+        if (wts) W += w;
+        P += in[k] ? w : 0;
       }
+    }
+    for (; j < j1; ++j) {
+      const int w = wts ? (int)wts[j] : 1;
+      if (wts) W += w;
+      P += get_bit(z, col[j], Bw, b) ? w : 0;
+    }
+    if (mis) {
+      a0 += zv;
+      a1 += zv ? P : 0;
+      a2 += !zv && P == 0;
+    } else {
       const int as = 2 * P - W;
       a0 += zv ? (W - P) : P;
       a1 += !(zv ? (as <= -1) : (as >= 0));
@@ -357,7 +391,8 @@ __global__ void __launch_bounds__(kPairThreads) k_eval(SolverDev S, const uint32
 }
 
 cudaError_t launch_eval(const SolverDev& S, const uint32_t* z, Counters* out, cudaStream_t stream) {
-  k_eval<<<S.g.num_items, kPairThreads, 0, stream>>>(S, z, out);
+  const SolverDev D = split_items(S, sm_count());
+  k_eval<<<D.g.num_items * D.split, kPairThreads, 0, stream>>>(D, z, out);
   return cudaGetLastError();
 }
 
@@ -389,31 +424,45 @@ cudaError_t launch_counters_out(const SolverDev& S, const Counters* c, int64_t* 
 // then the node's terms in double (MIS h; MaxCut f_B, f_L = 1/4 x'(D-A)x,
 // f_P = x'(D-A+lambda I)x or f_A = -x'Ax), accumulated per thread and
 // reduced per item in shared memory
+template <typename TX>
 __global__ void __launch_bounds__(kPairThreads) k_objective(SolverDev S, double* out) {
   __shared__ double s_obj[128];
   const int64_t t = *S.tick;
-  const void* Xc = (t & 1) ? S.X1 : S.X0;
+  const TX* __restrict__ Xc = static_cast<const TX*>((t & 1) ? S.X1 : S.X0);
+  const int32_t* __restrict__ rp = S.g.row_ptr;
+  const int32_t* __restrict__ col = S.g.col;
+  const int8_t* __restrict__ wts = S.g.w;
   const int B = S.B;
   const bool mis = S.p.problem == PROB_MIS;
-  auto ld = [&](int64_t e) -> float {
-    if (S.p.x_dtype == DT_F32) return static_cast<const float*>(Xc)[e];
-    if (S.p.x_dtype == DT_BF16) return __bfloat162float(static_cast<const __nv_bfloat16*>(Xc)[e]);
-    return __half2float(static_cast<const __half*>(Xc)[e]);
-  };
+  auto ld = [&](int64_t e) -> float { return to_f(Xc[e]); };
+  int it;
+  Item item;
+  if (!item_slice(S, it, item)) return;
   for (int i = threadIdx.x; i < B; i += blockDim.x) s_obj[i] = 0.0;
   __syncthreads();
-  const Item item = S.g.items[blockIdx.x];
   double part = 0.0;
   item_pairs(S, item, [&](const PairCtx& c) {
     if (!c.in) return;
+    const int32_t j1 = rp[c.v + 1];
+    int32_t j = rp[c.v];
     float acc = 0.0f;
-    int d = 0;
-    for (int32_t j = S.g.row_ptr[c.v]; j < S.g.row_ptr[c.v + 1]; ++j) {
-      const float xu = ld((int64_t)S.g.col[j] * B + c.b);
-      const int w = S.g.w == nullptr ? 1 : (int)S.g.w[j];
-      d += w;
-      if (w >= 0) acc = acc + xu;
-      else acc = acc - xu;
+    int d = wts ? 0 : j1 - j;
+    for (; j + kAhead <= j1; j += kAhead) {
+      float f[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) f[k] = ld((int64_t)col[j + k] * B + c.b);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int w = wts ? (int)wts[j + k] : 1;
+        if (wts) d += w;
+        acc = w >= 0 ? acc + f[k] : acc - f[k];
+      }
+    }
+    for (; j < j1; ++j) {
+      const float xu = ld((int64_t)col[j] * B + c.b);
+      const int w = wts ? (int)wts[j] : 1;
+      if (wts) d += w;
+      acc = w >= 0 ? acc + xu : acc - xu;
     }
     const double xv = (double)ld(c.v * B + c.b);
     const double xax = xv * (double)acc, lam = (double)S.p.lambda_;
@@ -435,8 +484,128 @@ __global__ void __launch_bounds__(kPairThreads) k_objective(SolverDev S, double*
     if (s_obj[i] != 0.0) atomicAdd(&out[(int64_t)item.g * B + i], s_obj[i]);
 }
 
+// The same with pieces of VEC values of x: a lane holds VEC
+// trajectories, B / VEC lanes a node, so one load serves 32 / (B / VEC) nodes; the
+// ids of a node's neighbours come one per lane and go round by shuffles.
+template <typename TX, int VEC, bool WEIGHTED>
+__global__ void __launch_bounds__(kPairThreads, 4) k_objective_v(SolverDev S, double* out) {
+  __shared__ double s_obj[128];
+  const int64_t t = *S.tick;
+  const TX* __restrict__ Xc = static_cast<const TX*>((t & 1) ? S.X1 : S.X0);
+  const int32_t* __restrict__ rp = S.g.row_ptr;
+  const int32_t* __restrict__ col = S.g.col;
+  const int8_t* __restrict__ wts = S.g.w;
+  const int B = S.B, lpr = B / VEC, rpw = 32 / lpr;
+  const bool mis = S.p.problem == PROB_MIS;
+  int it;
+  Item item;
+  if (!item_slice(S, it, item)) return;
+  for (int i = threadIdx.x; i < B; i += blockDim.x) s_obj[i] = 0.0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, sub = lane / lpr, l = lane - sub * lpr, warp = threadIdx.x >> 5;
+  const double lam = (double)S.p.lambda_;
+  double part[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) part[e] = 0.0;
+  for (int v0 = item.v0 + warp * rpw; v0 < item.v1; v0 += (kPairThreads / 32) * rpw) {
+    const int v = v0 + sub;
+    const bool in = v < item.v1;
+    const int32_t j0 = in ? rp[v] : 0, len = in ? rp[v + 1] - j0 : 0;
+    const int longest = __reduce_max_sync(0xffffffffu, len);
+    const Pack<TX, VEC> xv = ld_pack<TX, VEC>(Xc + (int64_t)(in ? v : item.v0) * B + l * VEC);
+    float acc[VEC];
+    int d = WEIGHTED ? 0 : len;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) acc[e] = 0.0f;
+    // ids (weights) of 4 lpr entries per round, one round ahead
+    int u[4], w[4], un[4], wn[4];
+    auto ids = [&](int k0, int* uu, int* ww) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int k = k0 + i * lpr + l;
+        uu[i] = k < len ? col[j0 + k] : -1;
+        if (WEIGHTED) ww[i] = k < len ? (int)wts[j0 + k] : 0;
+      }
+    };
+    ids(0, u, w);
+    for (int k0 = 0; k0 < longest; k0 += 4 * lpr) {
+      ids(k0 + 4 * lpr, un, wn);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        for (int k = 0; k < lpr && k0 + i * lpr + k < longest; k += 4) {
+          Pack<TX, VEC> p[4];
+          int uk[4], wk[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uk[q] = __shfl_sync(0xffffffffu, u[i], (k + q) & (lpr - 1), lpr);
+            if (WEIGHTED) wk[q] = __shfl_sync(0xffffffffu, w[i], (k + q) & (lpr - 1), lpr);
+            if (k + q >= lpr) uk[q] = -1;
+            if (uk[q] >= 0) p[q] = ld_pack<TX, VEC>(Xc + (int64_t)uk[q] * B + l * VEC);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (uk[q] < 0) continue;
+            if (WEIGHTED) d += wk[q];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e)
+              acc[e] = !WEIGHTED || wk[q] >= 0 ? acc[e] + to_f(p[q].e[e]) : acc[e] - to_f(p[q].e[e]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        u[i] = un[i];
+        if (WEIGHTED) w[i] = wn[i];
+      }
+    }
+    if (!in) continue;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      const double x = (double)to_f(xv.e[e]);
+      const double xax = x * (double)acc[e];
+      if (mis) {
+        part[e] += x - 0.5 * (double)S.p.gamma * xax;
+      } else {
+        const double xdx = (double)d * x * x;
+        switch (S.p.objective) {
+          case OBJ_FL: part[e] += 0.25 * (xdx - xax); break;
+          case OBJ_FP: part[e] += (xdx - xax) + lam * x * x; break;
+          case OBJ_FA: part[e] += -xax; break;
+          default: part[e] += -lam * x - xax; break;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) {
+    for (int o = lpr; o < 32; o <<= 1) part[e] += __shfl_xor_sync(0xffffffffu, part[e], o);
+    if (sub == 0 && part[e] != 0.0) atomicAdd(&s_obj[l * VEC + e], part[e]);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < B; i += blockDim.x)
+    if (s_obj[i] != 0.0) atomicAdd(&out[(int64_t)item.g * B + i], s_obj[i]);
+}
+
 cudaError_t launch_objective(const SolverDev& S, double* out, cudaStream_t stream) {
-  k_objective<<<S.g.num_items, kPairThreads, 0, stream>>>(S, out);
+  SolverDev D = split_items(S, sm_count());
+  constexpr int vec = 4;
+  if (S.B >= vec) D.split = std::max(1, std::min(D.split, S.B / vec));  // every warp of a CTA has rows
+  const int grid = D.g.num_items * D.split;
+  // (eight values per lane need more registers than four CTAs per SM have)
+  auto run = [&](auto tx) {
+    using TX = decltype(tx);
+    if (S.g.w) k_objective_v<TX, vec, true><<<grid, kPairThreads, 0, stream>>>(D, out);
+    else k_objective_v<TX, vec, false><<<grid, kPairThreads, 0, stream>>>(D, out);
+    return cudaGetLastError();
+  };
+  if (S.B >= vec) {
+    if (S.p.x_dtype == DT_F32) return run(float{});
+    if (S.p.x_dtype == DT_BF16) return run(__nv_bfloat16{});
+    return run(__half{});
+  }
+  if (S.p.x_dtype == DT_F32) k_objective<float><<<grid, kPairThreads, 0, stream>>>(D, out);
+  else if (S.p.x_dtype == DT_BF16) k_objective<__nv_bfloat16><<<grid, kPairThreads, 0, stream>>>(D, out);
+  else k_objective<__half><<<grid, kPairThreads, 0, stream>>>(D, out);
   return cudaGetLastError();
 }
 
