@@ -370,6 +370,18 @@ MQO_API mqo_status mqo_spmm_grad(mqo_graph g, const float* X, const float* gout,
                          void* cuda_stream);
 
 /*
+ * The two passes of a training step that share one product: the forward also
+ * writes AX[v*B+b] = (A X)_vb (float32, device, n*B, the sums both results are
+ * made of), and the backward forms the gradient of mqo_spmm_grad from it, bit for
+ * bit, without gathering again (one read and one write of n*B values).
+ * Arguments as mqo_fb_forward and mqo_spmm_grad.
+ */
+MQO_API mqo_status mqo_fb_forward_ax(mqo_graph g, const float* X, int32_t B, float lambda_, double* obj, float* AX,
+                                     void* cuda_stream);
+MQO_API mqo_status mqo_fb_grad_ax(mqo_graph g, const float* AX, const float* gout, float* G, int32_t B, float lambda_,
+                                  void* cuda_stream);
+
+/*
  * Same result as mqo_spmm_grad, but the call allocates nothing.  The paper
  * has no counterpart: this entry point exists for callers that cannot call
  * cudaMalloc during the call -- applications whose device memory is already

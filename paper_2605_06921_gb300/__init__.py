@@ -109,6 +109,8 @@ _SIGS = {
     "mqo_get_v": [_P, _P],
     "mqo_objective_f64": [_P, _P],
     "mqo_fb_forward": [_P, _P, C.c_int32, C.c_float, _P, _P],
+    "mqo_fb_forward_ax": [_P, _P, C.c_int32, C.c_float, _P, _P, _P],
+    "mqo_fb_grad_ax": [_P, _P, _P, _P, C.c_int32, C.c_float, _P],
     "mqo_spmm_grad": [_P, _P, _P, _P, C.c_int32, C.c_float, _P],
     "mqo_spmm_grad_static": [_P, _P, _P, _P, C.c_int32, C.c_float, _P],
     "mqo_pga_momentum_step": [_P, _P, _P, C.c_int64, C.c_float, C.c_float, C.c_float, C.c_float, _P],
@@ -420,18 +422,39 @@ def _autograd():
     import torch
 
     class FbObjective(torch.autograd.Function):
-        """f_B(X) per column (Eq. 7) with the fused SpMM gradient as backward."""
+        """f_B(X) per column (Eq. 7).  Where a gradient may be asked for, the
+        forward keeps A X and the backward forms the gradient from it (one
+        gather for both); X is saved too, so that a change of it in place
+        between the two is still an error."""
+
+        @classmethod
+        def apply(cls, X, graph, lambda_):
+            # the grad mode is off inside forward
+            return super().apply(X, graph, lambda_, torch.is_grad_enabled())
 
         @staticmethod
-        def forward(ctx, X, graph, lambda_):
+        def forward(ctx, X, graph, lambda_, grad_enabled):
             ctx.graph, ctx.lambda_ = graph, lambda_
-            ctx.save_for_backward(X)
-            return fb_forward(graph, X.detach(), lambda_)
+            if not (grad_enabled and ctx.needs_input_grad[0]):
+                return fb_forward(graph, X.detach(), lambda_)
+            Xc = X.detach().contiguous()
+            B = Xc.shape[1]
+            out = torch.empty(B, dtype=torch.float64, device=Xc.device)
+            ax = torch.empty_like(Xc)
+            _check(lib().mqo_fb_forward_ax(graph.handle, _dptr(Xc), B, float(lambda_), _dptr(out), _dptr(ax),
+                                           _stream()))
+            ctx.save_for_backward(X, ax)
+            return out
 
         @staticmethod
         def backward(ctx, gout):
-            (X,) = ctx.saved_tensors
-            return spmm_grad(ctx.graph, X.detach(), ctx.lambda_, gout), None, None
+            _, ax = ctx.saved_tensors
+            B = ax.shape[1]
+            G = torch.empty_like(ax)
+            g = gout.to(torch.float32).contiguous()
+            _check(lib().mqo_fb_grad_ax(ctx.graph.handle, _dptr(ax), _dptr(g), _dptr(G), B, float(ctx.lambda_),
+                                        _stream()))
+            return G, None, None, None
 
     class PGAMomentum(torch.optim.Optimizer):
         """Projected momentum ascent on p.grad: v <- mu v + g, p <- Pi(p + lr v)."""

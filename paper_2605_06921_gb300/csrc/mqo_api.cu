@@ -521,6 +521,12 @@ mqo_status build_heavy_plan(mqo_graph g) {
   // segments of consecutive light rows, cut before a heavy row or once a
   // segment holds kFbSegEntries entries
   std::vector<int32_t> segs;
+  for (size_t c = 0; c < hrow.size(); ++c) {
+    segs.push_back(hrow[c]);
+    segs.push_back(-1 - (int32_t)c);
+    segs.push_back(hj0[c]);
+    segs.push_back(hj1[c]);
+  }
   {
     int64_t r0 = -1;
     auto close = [&](int64_t r1) {
@@ -1516,8 +1522,10 @@ mqo_status mqo_objective_f64(mqo_solver s, double* out) {
   return MQO_OK;
 }
 
-mqo_status mqo_fb_forward(mqo_graph g, const float* X, int32_t B, float lambda_, double* obj, void* cuda_stream) {
-  if (!g || !X || !obj) return fail(MQO_EINVAL, "null argument");
+namespace {
+
+// Arguments of the f_B kernels: the chunk plan and its scratch, made on first use
+mqo_status fb_ready(mqo_graph g, const float* X, int32_t B) {
   if (B < 1 || B > 256 || (B & (B - 1))) return fail(MQO_EINVAL, "B=%d must be a power of two in [1,256]", B);
   // B >= 32: rows of X are read in 16-byte pieces
   if (B >= 32 && ((uintptr_t)X & 15u) != 0) return fail(MQO_EINVAL, "X must be 16-byte aligned for B >= 32");
@@ -1531,31 +1539,47 @@ mqo_status mqo_fb_forward(mqo_graph g, const float* X, int32_t B, float lambda_,
     if ((st = dalloc(&g->d_scratch, need, nullptr)) != MQO_OK) return st;
     g->scratch_floats = need;
   }
+  return MQO_OK;
+}
+
+}  // namespace
+
+mqo_status mqo_fb_forward(mqo_graph g, const float* X, int32_t B, float lambda_, double* obj, void* cuda_stream) {
+  if (!g || !X || !obj) return fail(MQO_EINVAL, "null argument");
+  const mqo_status st = fb_ready(g, X, B);
+  if (st != MQO_OK) return st;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   CKG(cudaMemsetAsync(obj, 0, sizeof(double) * B, s));
-  const int grid = g->sms * 8;
-  CKG(launch_fb(g->dev(), g->hp, X, B, lambda_, nullptr, nullptr, obj, g->d_scratch, grid, s));
+  CKG(launch_fb(g->dev(), g->hp, X, B, lambda_, nullptr, nullptr, nullptr, obj, g->d_scratch, g->sms * 8, s));
+  return MQO_OK;
+}
+
+mqo_status mqo_fb_forward_ax(mqo_graph g, const float* X, int32_t B, float lambda_, double* obj, float* AX,
+                             void* cuda_stream) {
+  if (!g || !X || !obj || !AX) return fail(MQO_EINVAL, "null argument");
+  const mqo_status st = fb_ready(g, X, B);
+  if (st != MQO_OK) return st;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  CKG(cudaMemsetAsync(obj, 0, sizeof(double) * B, s));
+  CKG(launch_fb(g->dev(), g->hp, X, B, lambda_, nullptr, nullptr, AX, obj, g->d_scratch, g->sms * 8, s));
+  return MQO_OK;
+}
+
+mqo_status mqo_fb_grad_ax(mqo_graph g, const float* AX, const float* gout, float* G, int32_t B, float lambda_,
+                          void* cuda_stream) {
+  if (!g || !AX || !G) return fail(MQO_EINVAL, "null argument");
+  if (B < 1 || B > 256 || (B & (B - 1))) return fail(MQO_EINVAL, "B=%d must be a power of two in [1,256]", B);
+  CKG(launch_grad_ax(AX, gout, G, g->n * B, B, lambda_, (cudaStream_t)cuda_stream));
   return MQO_OK;
 }
 
 mqo_status mqo_spmm_grad(mqo_graph g, const float* X, const float* gout, float* G, int32_t B, float lambda_,
                          void* cuda_stream) {
   if (!g || !X || !G) return fail(MQO_EINVAL, "null argument");
-  if (B < 1 || B > 256 || (B & (B - 1))) return fail(MQO_EINVAL, "B=%d must be a power of two in [1,256]", B);
-  // B >= 32: rows of X are read in 16-byte pieces
-  if (B >= 32 && ((uintptr_t)X & 15u) != 0) return fail(MQO_EINVAL, "X must be 16-byte aligned for B >= 32");
-  mqo_status st = build_heavy_plan(g);
+  const mqo_status st = fb_ready(g, X, B);
   if (st != MQO_OK) return st;
-  const size_t need = (size_t)g->hp.num_chunks * B;
-  if (need > g->scratch_floats) {
-    cudaFree(g->d_scratch);
-    g->d_scratch = nullptr;
-    g->scratch_floats = 0;
-    if ((st = dalloc(&g->d_scratch, need, nullptr)) != MQO_OK) return st;
-    g->scratch_floats = need;
-  }
-  const int grid = g->sms * 8;
-  CKG(launch_fb(g->dev(), g->hp, X, B, lambda_, gout, G, nullptr, g->d_scratch, grid, (cudaStream_t)cuda_stream));
+  CKG(launch_fb(g->dev(), g->hp, X, B, lambda_, gout, G, nullptr, nullptr, g->d_scratch, g->sms * 8,
+                (cudaStream_t)cuda_stream));
   return MQO_OK;
 }
 

@@ -22,8 +22,12 @@ namespace mqo {
 template <int VEC>
 struct FbOut {
   __device__ __forceinline__ static void emit(int64_t row, const float* acc, const float* X, int B, int b0,
-                                              float lambda_, const float* gout, float* G, bool want_obj,
+                                              float lambda_, const float* gout, float* G, float* AX, bool want_obj,
                                               float* objf) {
+    if (AX) {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) AX[row * B + b0 + e] = acc[e];
+    }
     if (G) {
       float o[VEC];
 #pragma unroll
@@ -57,6 +61,7 @@ struct FbArgs {
   float lambda_;
   const float* gout;
   float* G;
+  float* AX;  // (A X) itself, kept for a backward pass
   double* obj;
   float* scratch;
 };
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(256) k_fb_units(FbArgs a) {
       for (int e = 0; e < VEC; ++e) acc[e] = w >= 0 ? acc[e] + p.e[e] : acc[e] - p.e[e];
     }
     if (whole) {
-      FbOut<VEC>::emit(row, acc, a.X, B, b0, a.lambda_, a.gout, a.G, want_obj, objf);
+      FbOut<VEC>::emit(row, acc, a.X, B, b0, a.lambda_, a.gout, a.G, a.AX, want_obj, objf);
       if (++pending == 16) flush_obj<VEC>(objf, objd, pending);
     } else {
       const int64_t c = u - a.hp.num_light;
@@ -180,11 +185,12 @@ __global__ void __launch_bounds__(256) k_fb_heavy(FbArgs a) {
     float acc[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) acc[e] = 0.0f;
+#pragma unroll 8
     for (int32_t c = c0; c < c1; ++c) {
 #pragma unroll
       for (int e = 0; e < VEC; ++e) acc[e] = acc[e] + a.scratch[(int64_t)c * B + b0 + e];
     }
-    FbOut<VEC>::emit(row, acc, a.X, B, b0, a.lambda_, a.gout, a.G, want_obj, objf);
+    FbOut<VEC>::emit(row, acc, a.X, B, b0, a.lambda_, a.gout, a.G, a.AX, want_obj, objf);
     if (++pending == 16) flush_obj<VEC>(objf, objd, pending);
   }
   if (want_obj) {
@@ -227,9 +233,13 @@ __device__ __forceinline__ void fb_cp_async16(void* smem_dst, const void* gsrc) 
 // and batch i is summed.  Row ends come from a window of 32 row pointers
 // held across the lanes; every row is summed in CSR order and emitted as in
 // k_fb_units (gradient, objective), so the results equal k_fb_units's.
+// The 512-entry chunks of longer rows are segments too, the first ones, whose
+// sums go to scratch (as a kernel of their own they took 0.1 ms of the forward's
+// 0.5 ms on the power-law graph of 10^6 nodes, a few hundred chains of 512
+// gathers on an idle GPU).
 struct FbBatch {
   int64_t seg;  // segment index (>= num_segs: past the end)
-  int4 d;       // {first row, end row, first entry, end entry} of the segment
+  int4 d;       // {first row, end row, first entry, end entry} of the segment; a chunk: {row, -1 - chunk, ..}
   int32_t jb;   // first entry of the batch
 };
 
@@ -321,6 +331,10 @@ __global__ void __launch_bounds__(kFbPipeThreads) k_fb_seg(FbArgs a) {
     }
   };
   auto emit = [&]() {
+    if (a.AX) {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) __stcs(a.AX + (int64_t)row * B + b0 + e, acc[e]);
+    }
     if (a.G) {
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
@@ -363,9 +377,14 @@ __global__ void __launch_bounds__(kFbPipeThreads) k_fb_seg(FbArgs a) {
     int w3;
     load_idx(nx3, c3, w3);
     if (cur.jb == cur.d.z) {  // the first batch of a segment
-      seg_end_row = cur.d.y;
-      window(cur.d.x);
-      start_row(cur.d.x);
+      if (cur.d.y >= 0) {
+        seg_end_row = cur.d.y;
+        window(cur.d.x);
+        start_row(cur.d.x);
+      } else {  // a chunk: no row ends in it
+        row = seg_end_row = cur.d.x;
+        row_end = 0x7fffffff;
+      }
     }
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncwarp();
@@ -404,6 +423,14 @@ __global__ void __launch_bounds__(kFbPipeThreads) k_fb_seg(FbArgs a) {
     }
     __syncwarp();
     if (cur.jb + PIPE >= cur.d.w) {  // the segment's last batch: its remaining rows
+      if (cur.d.y < 0) {
+        const int64_t c = -1 - cur.d.y;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+          a.scratch[c * B + b0 + e] = acc[e];
+          acc[e] = 0.0f;
+        }
+      }
       while (row < seg_end_row) {
         emit();
         start_row(row + 1);
@@ -434,8 +461,8 @@ __global__ void __launch_bounds__(kFbPipeThreads) k_fb_seg(FbArgs a) {
 template <int VEC>
 static cudaError_t launch_fb_vec(const FbArgs& a, int grid, cudaStream_t s) {
   if (a.B == 32 * VEC && fb_pipe_enabled()) {
-    // light rows: the segment stream; heavy rows: their 512-entry chunks by
-    // the unit kernel, then the chunk sums
+    // light rows and the chunks of heavy rows: the segment stream; then the
+    // chunk sums
     if (a.hp.num_segs > 0) {
       constexpr int ROWB = 32 * VEC * 4;
       constexpr int PIPE = kFbPipeBytes / ROWB < 32 ? kFbPipeBytes / ROWB : 32;
@@ -454,11 +481,6 @@ static cudaError_t launch_fb_vec(const FbArgs& a, int grid, cudaStream_t s) {
       const cudaError_t e = a.g.w ? run(k_fb_seg<VEC, true>) : run(k_fb_seg<VEC, false>);
       if (e != cudaSuccess) return e;
     }
-    if (a.hp.num_chunks > 0) {
-      FbArgs c = a;
-      c.hp.num_light = 0;  // units = the chunks of heavy rows only
-      k_fb_units<VEC><<<grid, 256, 0, s>>>(c);
-    }
   } else if ((int64_t)a.hp.num_light + a.hp.num_chunks > 0) {
     k_fb_units<VEC><<<grid, 256, 0, s>>>(a);
   }
@@ -467,8 +489,9 @@ static cudaError_t launch_fb_vec(const FbArgs& a, int grid, cudaStream_t s) {
 }
 
 cudaError_t launch_fb(const GraphDev& g, const HeavyPlan& hp, const float* X, int B, float lambda_,
-                      const float* gout, float* G, double* obj, float* scratch, int grid, cudaStream_t stream) {
-  FbArgs a{g, hp, X, B, lambda_, gout, G, obj, scratch};
+                      const float* gout, float* G, float* AX, double* obj, float* scratch, int grid,
+                      cudaStream_t stream) {
+  FbArgs a{g, hp, X, B, lambda_, gout, G, AX, obj, scratch};
   const int vec = B >= 32 ? B / 32 : 1;
   switch (vec) {
     case 1: return launch_fb_vec<1>(a, grid, stream);
@@ -479,45 +502,108 @@ cudaError_t launch_fb(const GraphDev& g, const HeavyPlan& hp, const float* X, in
   }
 }
 
-// ---------------------------------------------------------------- optimisers
-__global__ void k_momentum(float* x, float* v, const float* grad, int64_t n, float lr, float mu, float lo, float hi) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float a = mu * v[i];
-    const float vn = a + grad[i];
-    v[i] = vn;
-    const float step = lr * vn;
-    x[i] = clamp_box(x[i] + step, lo, hi);
+// ---------------------------------------------------------------- elementwise
+// The kernels below stream their arrays once and are bound by DRAM; where every
+// array is on a 16-byte boundary a thread takes four elements at a time
+// (momentum on 64 M elements: 0.28 ms element by element, 0.21 ms; 1.28 GB).
+static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+static int stream_grid(int64_t threads) { return (int)std::max<int64_t>(1, std::min<int64_t>((threads + 255) / 256, 152 * 16)); }
+
+// gradient from a kept A X: G = gout (-lambda - 2 A X), rounded as in emit
+template <int V>
+__global__ void __launch_bounds__(256) k_grad_ax(const float* __restrict__ AX, const float* __restrict__ gout,
+                                                 float* __restrict__ G, int64_t n, int B, float lambda_) {
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V; i < n; i += (int64_t)gridDim.x * blockDim.x * V) {
+    Pack<float, V> p = ld_pack_stream<float, V>(AX + i);
+    const int b = (int)(i & (B - 1));  // B is a power of two, V divides it
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      const float tt = 2.0f * p.e[e];
+      float gr = -lambda_ - tt;
+      if (gout) gr = gout[b + e] * gr;
+      p.e[e] = gr;
+    }
+    st_pack<float, V>(G + i, p);
   }
 }
 
-__global__ void k_adam(float* x, float* m, float* u, const float* grad, int64_t n, float lr, float b1, float b2,
-                       float eps, float c1, float c2, float lo, float hi) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float g = grad[i];
-    const float mn = b1 * m[i] + (1.0f - b1) * g;
-    const float un = b2 * u[i] + (1.0f - b2) * (g * g);
-    m[i] = mn;
-    u[i] = un;
+cudaError_t launch_grad_ax(const float* AX, const float* gout, float* G, int64_t n, int B, float lambda_,
+                           cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (B % 4 == 0 && aligned16(AX) && aligned16(G)) k_grad_ax<4><<<stream_grid(n / 4), 256, 0, s>>>(AX, gout, G, n, B, lambda_);
+  else k_grad_ax<1><<<stream_grid(n), 256, 0, s>>>(AX, gout, G, n, B, lambda_);
+  return cudaGetLastError();
+}
+
+// elements [0, n) by V at a time; the n % V last ones by the first threads
+template <int V>
+__global__ void __launch_bounds__(256) k_momentum(float* x, float* v, const float* grad, int64_t n, float lr, float mu,
+                                                  float lo, float hi) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  auto one = [&](float xi, float& vi, float gi) {
+    const float a = mu * vi;
+    vi = a + gi;
+    const float step = lr * vi;
+    return clamp_box(xi + step, lo, hi);
+  };
+  for (int64_t i = t * V; i + V <= n; i += (int64_t)gridDim.x * blockDim.x * V) {
+    Pack<float, V> px = ld_pack<float, V>(x + i), pv = ld_pack<float, V>(v + i);
+    const Pack<float, V> pg = ld_pack_stream<float, V>(grad + i);
+#pragma unroll
+    for (int e = 0; e < V; ++e) px.e[e] = one(px.e[e], pv.e[e], pg.e[e]);
+    st_pack<float, V>(v + i, pv);
+    st_pack<float, V>(x + i, px);
+  }
+  const int64_t i = n - n % V + t;
+  if (V > 1 && i < n) x[i] = one(x[i], v[i], grad[i]);
+}
+
+template <int V>
+__global__ void __launch_bounds__(256) k_adam(float* x, float* m, float* u, const float* grad, int64_t n, float lr,
+                                              float b1, float b2, float eps, float c1, float c2, float lo, float hi) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  auto one = [&](float xi, float& mi, float& ui, float g) {
+    const float mn = b1 * mi + (1.0f - b1) * g;
+    const float un = b2 * ui + (1.0f - b2) * (g * g);
+    mi = mn;
+    ui = un;
     const float mh = mn * c1;
     const float uh = un * c2;
     const float step = lr * mh / (sqrtf(uh) + eps);
-    x[i] = clamp_box(x[i] + step, lo, hi);
+    return clamp_box(xi + step, lo, hi);
+  };
+  for (int64_t i = t * V; i + V <= n; i += (int64_t)gridDim.x * blockDim.x * V) {
+    Pack<float, V> px = ld_pack<float, V>(x + i), pm = ld_pack<float, V>(m + i), pu = ld_pack<float, V>(u + i);
+    const Pack<float, V> pg = ld_pack_stream<float, V>(grad + i);
+#pragma unroll
+    for (int e = 0; e < V; ++e) px.e[e] = one(px.e[e], pm.e[e], pu.e[e], pg.e[e]);
+    st_pack<float, V>(m + i, pm);
+    st_pack<float, V>(u + i, pu);
+    st_pack<float, V>(x + i, px);
   }
+  const int64_t i = n - n % V + t;
+  if (V > 1 && i < n) x[i] = one(x[i], m[i], u[i], grad[i]);
 }
 
 cudaError_t launch_momentum(float* x, float* v, const float* grad, int64_t n, float lr, float mu, float lo,
                             float hi, cudaStream_t stream) {
-  const int grid = (int)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16);
-  if (n > 0) k_momentum<<<grid, 256, 0, stream>>>(x, v, grad, n, lr, mu, lo, hi);
+  if (n <= 0) return cudaSuccess;
+  if (aligned16(x) && aligned16(v) && aligned16(grad))
+    k_momentum<4><<<stream_grid(n / 4 + 1), 256, 0, stream>>>(x, v, grad, n, lr, mu, lo, hi);
+  else
+    k_momentum<1><<<stream_grid(n), 256, 0, stream>>>(x, v, grad, n, lr, mu, lo, hi);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adam(float* x, float* m, float* u, const float* grad, int64_t n, float lr, float b1, float b2,
                         float eps, int64_t t, float lo, float hi, cudaStream_t stream) {
-  const int grid = (int)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16);
+  if (n <= 0) return cudaSuccess;
   const float c1 = (float)(1.0 / (1.0 - pow((double)b1, (double)t)));
   const float c2 = (float)(1.0 / (1.0 - pow((double)b2, (double)t)));
-  if (n > 0) k_adam<<<grid, 256, 0, stream>>>(x, m, u, grad, n, lr, b1, b2, eps, c1, c2, lo, hi);
+  if (aligned16(x) && aligned16(m) && aligned16(u) && aligned16(grad))
+    k_adam<4><<<stream_grid(n / 4 + 1), 256, 0, stream>>>(x, m, u, grad, n, lr, b1, b2, eps, c1, c2, lo, hi);
+  else
+    k_adam<1><<<stream_grid(n), 256, 0, stream>>>(x, m, u, grad, n, lr, b1, b2, eps, c1, c2, lo, hi);
   return cudaGetLastError();
 }
 

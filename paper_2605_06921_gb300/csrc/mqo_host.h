@@ -89,8 +89,9 @@ struct HeavyPlan {
   const int32_t* heavy_rows;  // distinct heavy rows
   const int32_t* heavy_first; // per heavy row: first chunk
   int32_t num_heavy;
-  // light rows in segments of consecutive rows (no heavy row inside) of
-  // about kFbSegEntries entries: {first row, end row, first entry, end entry}
+  // the chunks, {row, -1 - chunk, first entry, end entry}, then the light rows in
+  // segments of consecutive rows (no heavy row inside) of about kFbSegEntries
+  // entries: {first row, end row, first entry, end entry}
   const int4* segs;
   int32_t num_segs;
 };
@@ -102,7 +103,10 @@ cudaError_t launch_smem_probe(int grid, int32_t iters, uint32_t* sink, cudaStrea
 int smem_probe_threads();
 
 cudaError_t launch_fb(const GraphDev& g, const HeavyPlan& hp, const float* X, int B, float lambda_,
-                      const float* gout, float* G, double* obj, float* scratch, int grid, cudaStream_t stream);
+                      const float* gout, float* G, float* AX, double* obj, float* scratch, int grid,
+                      cudaStream_t stream);
+cudaError_t launch_grad_ax(const float* AX, const float* gout, float* G, int64_t n, int B, float lambda_,
+                           cudaStream_t s);
 cudaError_t launch_momentum(float* x, float* v, const float* grad, int64_t n, float lr, float mu, float lo,
                             float hi, cudaStream_t stream);
 cudaError_t launch_adam(float* x, float* m, float* u, const float* grad, int64_t n, float lr, float b1, float b2,
