@@ -49,7 +49,7 @@ def _plan(p):
     if p & 1:
         kern = "smem_wide" if p & 4 else "smem"
     else:
-        kern = "staged" if p & 8 else "global"
+        kern = "staged" if p & 8 else "rows" if p & (1 << 20) else "global"
     return {"step_kernel": kern, "discrete_kernel": "graph" if p & 2 else "pairs", "lanes_vec": (p >> 4) & 15,
             "slice_kb": (p >> 8) & 255, "col16": bool(p & (1 << 16)), "ell": bool(p & (1 << 17)),
             "dense": bool(p & (1 << 18)), "small": bool(p & (1 << 19))}

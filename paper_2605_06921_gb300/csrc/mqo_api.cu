@@ -118,6 +118,7 @@ struct mqo_solver_s {
   bool poisoned = false;
   size_t step_smem = 0;  // > 0: shared-memory step kernel with this much dynamic smem
   size_t disc_smem = 0;  // > 0: fused per-graph discrete kernel with this much dynamic smem
+  bool rows_ok = false;      // the row-group step kernel is possible
   size_t step_smem_max = 0;  // smem the shared-memory step kernel needs (0: not possible)
   size_t disc_smem_max = 0;  // smem the fused discrete kernel needs (0: not possible)
   size_t disc_bits_max = 0;  // smem of its form on bit matrices (0: not possible)
@@ -742,13 +743,13 @@ cudaError_t enqueue_tick(mqo_solver s) {
       for (int pass = 0; pass < 3; ++pass)
         if ((e = launch_disc(S, pass, s->work2)) != cudaSuccess) return e;
     }
-    if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense)) != cudaSuccess)
+    if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense, s->g->sms)) != cudaSuccess)
       return e;
     if ((e = cudaEventRecord(s->ev_join, s->work2)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(s->work, s->ev_join, 0)) != cudaSuccess) return e;
     return launch_tick_end(S, s->work);
   }
-  if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense)) != cudaSuccess) return e;
+  if ((e = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense, s->g->sms)) != cudaSuccess) return e;
   if (s->disc_smem > 0) {
     if ((e = launch_disc_fused(s, s->work)) != cudaSuccess) return e;
   } else {
@@ -1050,6 +1051,13 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         s->small = tk ? strcmp(tk, "small") == 0 : !other && faster;
       }
     }
+    // MaxCut on f_B with 16-bit x outside shared memory: the row-group kernel
+    // (MQO_STEP_KERNEL=rows: also where the member graphs fit in shared memory).
+    s->rows_ok = step_rows_possible(B, p->x_dtype, p->problem, p->objective, g->max_deg);
+    if (s->rows_ok && ((!force && s->step_smem == 0 && !s->dense) || (force && strcmp(force, "rows") == 0))) {
+      s->step_smem = 0;
+      s->S.step_staged = 2;
+    }
     if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
     // The fused per-graph discrete kernel runs one CTA per member graph, so
     // it is the default only with at least half as many member graphs as
@@ -1196,7 +1204,7 @@ mqo_status mqo_run_timed(mqo_solver s, int64_t nticks, double* phase_ms, int64_t
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
       if (ek == cudaSuccess) ek = launch_apply(S, s->work);
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
-      if (ek == cudaSuccess) ek = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense);
+      if (ek == cudaSuccess) ek = launch_step(S, S.cnt, S.act, S.gflag + 2 * G, s->step_smem, s->work, s->ell, s->ell_pos, s->dense, s->g->sms);
       if (ek == cudaSuccess) ek = cudaEventRecordWithFlags(e[i++], s->work, cudaEventRecordExternal);
       for (int pass = 0; pass < 3 && ek == cudaSuccess; ++pass) {
         if (s->disc_smem > 0) {
@@ -1256,7 +1264,7 @@ mqo_status mqo_step(mqo_solver s, int32_t nsteps) {
   }
   for (int32_t i = 0; i < nsteps; ++i) {
     CKS(cudaMemsetAsync(s->d_cnt_plain, 0, sizeof(Counters) * (size_t)S.g.num_graphs * S.B * S.R, s->work));
-    CKS(launch_step(S, s->d_cnt_plain, nullptr, nullptr, s->step_smem, s->work, s->ell, s->ell_pos, s->dense));
+    CKS(launch_step(S, s->d_cnt_plain, nullptr, nullptr, s->step_smem, s->work, s->ell, s->ell_pos, s->dense, s->g->sms));
     CKS(launch_tick_end(S, s->work));
   }
   s->host_tick += nsteps;
@@ -1378,9 +1386,11 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                            int32_t* replicas) {
   if (!s) return fail(MQO_EINVAL, "null solver");
   const int B = s->S.B;
-  const bool staged = s->step_smem == 0 && s->S.step_staged && !s->dense;
+  const bool staged = s->step_smem == 0 && s->S.step_staged == 1 && !s->dense;
+  const bool rows = s->step_smem == 0 && s->S.step_staged == 2 && !s->dense;
   const bool smem = s->step_smem > 0 || s->dense;
-  const int vec = smem ? 0
+  const int vec = smem   ? 0
+                  : rows ? 8
                   : (s->S.step_vec > 0 ? s->S.step_vec
                                        : (staged ? default_staged_vec(B, s->S.p.x_dtype)
                                                  : default_step_vec(B, s->S.p.x_dtype)));
@@ -1390,7 +1400,7 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                    ((staged ? slice_kb(s) : 0) << 8) |
                    ((s->step_smem > 0 && s->S.step_c16 && !s->dense) ? (1 << 16) : 0) |
                    ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0) |
-                   (s->small ? (1 << 19) : 0);
+                   (s->small ? (1 << 19) : 0) | (rows ? (1 << 20) : 0);
   if (smem_bytes) *smem_bytes = (int64_t)(s->dense ? s->dense->smem : s->step_smem);
   if (items) *items = s->S.g.num_items;
   if (replicas) *replicas = s->S.R;
@@ -1659,7 +1669,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     int vec;
     int wide;
     size_t disc_smem;
-    int staged;   // staged-gather step kernel
+    int staged;   // 1: staged-gather step kernel, 2: row groups
     int slice_kb; // its slice capacity
     int c16;      // shared-memory step kernel with 16-bit column indices
     int ell;      // shared-memory step kernel with the sliced-ELL stream
@@ -1697,6 +1707,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
             for (int v : {2, 4, 8})
               if (staged_vec_ok(B, S.p.x_dtype, v)) plans.push_back({0, v, 0, dc, 1, kb, 0, 0, 0});
           }
+        if (s->rows_ok) plans.push_back({0, 0, 0, dc, 2, 0, 0, 0, 0});
       }
     }
   if (s->dense_ok)
@@ -1752,7 +1763,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
       s->disc_bits = pl.dbits != 0;
       S.step_staged = pl.staged;
       S.step_c16 = pl.c16;
-      if (pl.staged) use_slices(s, slice_set(s, pl.slice_kb));
+      if (pl.staged == 1) use_slices(s, slice_set(s, pl.slice_kb));
       use_ell(s, pl.step_smem > 0 && pl.ell);
       s->dense = pl.dense ? &s->dense_plan : nullptr;
       if (pl.ell && !s->step_ell) continue;  // its arrays could not be built
@@ -1807,13 +1818,15 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
   if (s->gx16) cudaGraphExecDestroy(s->gx16);
   s->gx1 = s->gx16 = nullptr;
   if (plan_out) {
-    const bool stg = chosen.step_smem == 0 && chosen.staged && !chosen.dense;
+    const bool stg = chosen.step_smem == 0 && chosen.staged == 1 && !chosen.dense;
+    const bool rows = chosen.step_smem == 0 && chosen.staged == 2 && !chosen.dense;
+    if (rows) chosen.vec = 8;
     if (chosen.dense) chosen.wide = chosen.c16 = chosen.ell = chosen.vec = 0;
     *plan_out = (chosen.step_smem > 0 || chosen.dense ? 1 : 0) | (chosen.dense ? (1 << 18) : 0) |
                 (chosen.small ? (1 << 19) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
                 (stg ? 8 : 0) | (chosen.vec << 4) | ((stg ? chosen.slice_kb : 0) << 8) |
                 ((chosen.step_smem > 0 && chosen.c16) ? (1 << 16) : 0) |
-                ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0);
+                ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0) | (rows ? (1 << 20) : 0);
   }
   if (best_ms_per_tick) *best_ms_per_tick = best / ticks;
   return MQO_OK;

@@ -137,7 +137,7 @@ struct SolverDev {
   int32_t step_wide; // shared-memory step kernel with 16-byte lanes
   int32_t step_c16;  // shared-memory step kernel reads the 16-bit member-local column indices
   int32_t split;    // CTAs per item of the node-parallel kernels (several when there are few items)
-  int32_t step_staged;  // 1: staged-gather step kernel (when the shared-memory one is not used)
+  int32_t step_staged;  // when the shared-memory step kernel is not used: 1 staged-gather, 2 row groups, 0 global
   const Slice* slices;  // its slices, their count, and the most rows / CSR entries of one slice
   int32_t num_slices, slice_rows, slice_cols;
   void* X0;         // relaxed x: tick t reads X[t&1] and writes X[(t+1)&1]

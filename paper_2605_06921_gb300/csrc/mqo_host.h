@@ -17,8 +17,8 @@ struct DensePlan;
 // with the sliced-ELL neighbour stream when `ell` is given (build_ell);
 // `dense`: the tensor-core kernel of dense member graphs instead
 cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, const int32_t* gflag_step,
-                        size_t smem, cudaStream_t stream, const int4* ell = nullptr, const int2* ell_pos = nullptr,
-                        const DensePlan* dense = nullptr);
+                        size_t smem, cudaStream_t stream, const int4* ell, const int2* ell_pos,
+                        const DensePlan* dense, int sms);
 // the sliced-ELL stream of the shared-memory step kernel (mqo_step_smem.cuh)
 // for `rpw` rows per warp and x rows `pitch` bytes apart, from the group
 // table `pos` (one entry per processing position)
@@ -37,6 +37,8 @@ cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const 
                               uint4* bits, cudaStream_t s);
 size_t dense_smem_bytes(int max_ng);
 bool step_wide_possible(int B, int x_dtype);
+// the row-group kernel of MaxCut on f_B (mqo_step_rows.cu)
+bool step_rows_possible(int B, int x_dtype, int problem, int objective, int max_degree);
 int default_step_vec(int B, int x_dtype);
 bool staged_vec_ok(int B, int x_dtype, int vec);
 int default_staged_vec(int B, int x_dtype);

@@ -2,7 +2,8 @@
 // (mqo_step_smem.cuh; here with column indices from the CSR arrays, in
 // mqo_step_ell.cu with the sliced-ELL stream), the tensor-core kernel of dense
 // member graphs (mqo_step_dense.cuh), the staged-gather kernel
-// (mqo_step_staged.cu) or the global-memory kernel (mqo_step_generic.cu).
+// (mqo_step_staged.cu), the row-group kernel (mqo_step_rows.cu) or the
+// global-memory kernel (mqo_step_generic.cu).
 // The step itself (gradient, momentum, projection, rounding, exact
 // evaluation) is described in mqo_step.cuh.
 #include "mqo_step_dense.cuh"
@@ -13,6 +14,9 @@ namespace mqo {
 // the shared-memory kernel with the sliced-ELL stream (mqo_step_ell.cu)
 cudaError_t launch_smem_ell(const StepArgs& a, bool wide, size_t smem, bool mis, const int4* ell, const int2* ell_pos,
                             int grid, int x_dtype, int v_dtype, cudaStream_t s);
+
+// the row-group kernel (mqo_step_rows.cu)
+cudaError_t launch_step_rows(const StepArgs& a, int x_dtype, int v_dtype, int sms, cudaStream_t s);
 
 size_t step_smem_bytes(int B, int x_dtype, int problem, int max_ng) {
   const size_t sx = x_dtype == DT_F32 ? 4 : 2;
@@ -31,7 +35,8 @@ static cudaError_t launch_tv(bool wide, size_t smem, bool mis, const StepArgs& a
 }
 
 cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, const int32_t* gflag_step,
-                        size_t smem, cudaStream_t stream, const int4* ell, const int2* ell_pos, const DensePlan* dense) {
+                        size_t smem, cudaStream_t stream, const int4* ell, const int2* ell_pos, const DensePlan* dense,
+                        int sms) {
   StepArgs a;
   a.g = S.g;
   a.B = S.B;
@@ -60,6 +65,7 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
   a.slice_cols = S.slice_cols;
   const int xd = S.p.x_dtype, vd = S.p.v_dtype;
   if (dense) return launch_step_dense(a, *dense, S.any + 3, xd, vd, stream);
+  if (smem == 0 && S.step_staged == 2) return launch_step_rows(a, xd, vd, sms, stream);
   if (smem == 0 && S.step_staged) {
     // staged-gather kernel: one CTA per slice
     const int vec = S.step_vec > 0 ? S.step_vec : default_staged_vec(S.B, xd);
