@@ -43,6 +43,7 @@ constexpr size_t kSmallSmemLimit = 200 * 1024;  // multi-tick kernel: a member g
 constexpr int kSmallTicks = 4096;               // ticks per launch of that kernel
 constexpr int kDenseMaxDegree = 1023;  // tensor-core step: neighbour counts take 10 bits
 constexpr size_t kDenseSmemLimit = 225 * 1024;  // and 32 trajectories of a member graph's x fit in shared memory
+constexpr int64_t kL2Bytes = (int64_t)129 << 20;
 constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3 bytes per CSR entry at most)
 constexpr int kDefaultSliceKB = 32;  // staged step kernel: gathered x rows per slice (KB)
 
@@ -1051,12 +1052,40 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         s->small = tk ? strcmp(tk, "small") == 0 : !other && faster;
       }
     }
-    // MaxCut on f_B with 16-bit x outside shared memory: the row-group kernel
-    // (MQO_STEP_KERNEL=rows: also where the member graphs fit in shared memory).
+    // 16-bit x, MIS or MaxCut on f_B: the row-group kernel, unless an environment
+    // variable selects one of the others (MQO_STEP_KERNEL=rows: this one where
+    // possible).  A row's neighbours are read a few at a time, so the longest row
+    // is a chain of L2 latencies (about 0.15 us per entry beyond what the staged
+    // kernel takes), to be covered by the time of the whole step at about 5 TB/s of
+    // L2 reads.  Measured, rows against staged: n = 10^4, degree 20 (longest 40),
+    // B = 32 23.7 us against 19.7, B = 64 23.6 against 25.5, B = 128 29 against 36;
+    // n = 5 10^4, longest row 864, B = 32: 227 against 30.  Rows of 64 bytes from an
+    // x far larger than L2 wait for DRAM, which the staged kernel's deeper queue
+    // serves better (10^7 nodes, B = 32: 3.25 ms against 3.42; 4 10^6: the same).
     s->rows_ok = step_rows_possible(B, p->x_dtype, p->problem, p->objective, g->max_deg);
-    if (s->rows_ok && ((!force && s->step_smem == 0 && !s->dense) || (force && strcmp(force, "rows") == 0))) {
-      s->step_smem = 0;
-      s->S.step_staged = 2;
+    const bool none_forced = !force && !ellv && !c16;
+    {
+      const bool covered = (double)(g->nnz + 4 * g->n) * B >= 375e3 * g->max_deg;
+      const bool dram = B == 32 && g->n * B * 2 > 2 * kL2Bytes && p->v_dtype != DT_F32;
+      bool rows = s->rows_ok && covered && !dram;
+      if (none_forced && s->step_smem > 0) {
+        // Member graphs that fit in shared memory: that kernel runs one CTA per item
+        // and leaves the GPU idle below about a third as many items as SMs (n = 300,
+        // degree 20, B = 128, MIS: 8 items 34 us against 15 of the staged kernel, 32
+        // items 35 against 23, 100 items 35 against 41).  MaxCut's longer tail moves
+        // its line against the row groups to as many items as SMs, or to a mean degree
+        // of 8 (B = 128: 100 items, degree 20: 53 against 34; 300 items, degree 4: 49
+        // against 38, degree 20: 74 against 76).
+        const int items = (int)g->h_items.size();
+        const bool few = 3 * items < g->sms && (s->staged_ok || rows);
+        const bool cut = p->problem == PROB_MAXCUT && rows && (items < g->sms || g->nnz <= 8 * g->n);
+        if (few || cut) s->step_smem = 0;
+        else rows = false;
+      }
+      if ((none_forced && rows && !s->dense) || (s->rows_ok && force && strcmp(force, "rows") == 0)) {
+        s->step_smem = 0;
+        s->S.step_staged = 2;
+      }
     }
     if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
     // The fused per-graph discrete kernel runs one CTA per member graph, so
@@ -1821,6 +1850,8 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     const bool stg = chosen.step_smem == 0 && chosen.staged == 1 && !chosen.dense;
     const bool rows = chosen.step_smem == 0 && chosen.staged == 2 && !chosen.dense;
     if (rows) chosen.vec = 8;
+    else if (chosen.step_smem == 0 && !chosen.dense && chosen.vec == 0)
+      chosen.vec = stg ? default_staged_vec(B, S.p.x_dtype) : default_step_vec(B, S.p.x_dtype);
     if (chosen.dense) chosen.wide = chosen.c16 = chosen.ell = chosen.vec = 0;
     *plan_out = (chosen.step_smem > 0 || chosen.dense ? 1 : 0) | (chosen.dense ? (1 << 18) : 0) |
                 (chosen.small ? (1 << 19) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |

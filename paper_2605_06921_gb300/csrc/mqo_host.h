@@ -37,7 +37,7 @@ cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const 
                               uint4* bits, cudaStream_t s);
 size_t dense_smem_bytes(int max_ng);
 bool step_wide_possible(int B, int x_dtype);
-// the row-group kernel of MaxCut on f_B (mqo_step_rows.cu)
+// the row-group kernel (mqo_step_rows.cu)
 bool step_rows_possible(int B, int x_dtype, int problem, int objective, int max_degree);
 int default_step_vec(int B, int x_dtype);
 bool staged_vec_ok(int B, int x_dtype, int vec);

@@ -1,22 +1,27 @@
-// mqo_step_rows.cu -- the fused descent step of MaxCut (f_B) with 16-bit x on
-// graphs too large for shared memory (k_step_r).  The step itself (gradient,
-// momentum, projection, rounding, exact evaluation) is the one of mqo_step.cuh.
+// mqo_step_rows.cu -- the fused descent step with 16-bit x, for MIS and for
+// MaxCut on f_B, reading neighbour rows straight from L2 (k_step_r).  The step
+// itself (gradient, momentum, projection, rounding, exact evaluation) is the
+// one of mqo_step.cuh.
 //
-// Why: on the 3-regular graph (n = 10^5, B = 128) x stays in L2 and the staged
-// kernel is bound by issue: 140 lane instructions per (node, trajectory) pair,
-// most of them in the per-element tail, 79 us.  Here a lane holds 8
-// trajectories in four words and works on words:
+// Why: while x stays in L2 the staged kernel is bound by issue, 140 lane
+// instructions per (node, trajectory) pair of degree 3, most of them in the
+// per-element tail.  Here a lane holds 8 trajectories in four words and works
+// on words:
 //  * a neighbour adds its four words to the sums with mixed-precision adds (one
 //    rounding each, CSR order) and its four "in the set" masks to packed 16-bit
-//    counts;
-//  * with Q the number of neighbours on the set's side (for a weight of -1 the
-//    other side counts), As = 2 Q - d, so the fixed-point and gain tests are
-//    one packed add and one logic operation per word;
+//    counts (MIS: to an OR);
+//  * MaxCut: with Q the number of neighbours on the set's side (for a weight of
+//    -1 the other side counts), As = 2 Q - d, so the fixed-point and gain tests
+//    are one packed add and one logic operation per word;
 //  * the cut needs only the set's own nodes: summed over a symmetric graph,
 //    sum_v [z_v ? W_v - P_v : P_v] = 2 sum_{z_v = 1} (W_v - P_v).
-// A row group of B / 8 lanes takes one row; its neighbour rows are gathered
-// with 16-byte loads, four in flight (L2, no staging: a row of degree 3 has
-// nothing to pipeline).  About 25 lane instructions per pair of degree 3.
+// A row group of B / 8 lanes takes one row and gathers its neighbours' rows
+// with 16-byte loads, three in flight.  Bound by the L2 path and its latency at
+// 64 registers (32 warps per SM, one wave of CTAs).  Measured (step, degree 3,
+// B = 128, MaxCut, BF16): n = 10^5 41 us against 79 of the staged kernel and 80
+// of the global-memory one, FP32 V 48 against 103 and 83; n = 10^6 403 against
+// 668; n = 10^5, degree 16: 92 against 210 and 185, MIS 85 against 182 and 185.
+// Four or eight rows in flight take 43 and 61 us, 48 or 80 registers 49 and 55.
 #include "mqo_step.cuh"
 #include "mqo_x16.cuh"
 
@@ -25,6 +30,7 @@ namespace mqo {
 namespace {
 
 constexpr int kRowThreads = 256;
+constexpr int kRowDepth = 3;    // neighbour rows in flight per lane
 constexpr int kRowCols = 2048;  // staged column indices per CTA; longer lists are read from global memory
 
 // (a, b) = (a, b) * (x, x) + (y, y), one rounding
@@ -43,7 +49,7 @@ __device__ __forceinline__ void fma2(float& a, float& b, float x, float y) {
 
 // CTA c takes rows [c * per, (c + 1) * per) of the one member graph (per > 0),
 // or part c % split of item c / split (per == 0); at most kItemMaxNodes rows
-template <typename TX, typename TV, bool WEIGHTED>
+template <typename TX, typename TV, bool MIS, bool WEIGHTED>
 __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) {
   using X = X16<TX>;
   using T2 = typename X::T2;
@@ -92,9 +98,10 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
   for (int e = 0; e < 8; ++e)
     stepm |= (uint32_t)(a.act ? (a.act[(int64_t)g * B + b0 + e] & ACT_STEP) != 0 : true) << e;
   const bool all_step = __all_sync(0xffffffffu, stepm == 0xffu);
-  const T2 zero2 = X::splat(0.0f), one2 = X::splat(1.0f), low2 = X::splat(-1.0f);
-  // packed 16-bit sums over the lane's rows: of a set node's d - (negative
-  // entries) and Q, of nodes not fixed and of nodes with a positive gain
+  const T2 thr2 = X::splat(MIS ? 0.5f : 0.0f), one2 = X::splat(1.0f), low2 = X::splat(MIS ? 0.0f : -1.0f);
+  // packed 16-bit sums over the lane's rows.  MaxCut: of a set node's d -
+  // (negative entries) and Q, of nodes not fixed and of nodes with a positive
+  // gain; MIS: zd of nodes in the set, n1 of those in conflict, n2 of uncovered
   uint32_t zd[4], zq[4], n1[4], n2[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) zd[i] = zq[i] = n1[i] = n2[i] = 0u;
@@ -116,15 +123,15 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
       vf[0] = q0.x, vf[1] = q0.y, vf[2] = q0.z, vf[3] = q0.w, vf[4] = q1.x, vf[5] = q1.y, vf[6] = q1.z, vf[7] = q1.w;
     }
     float acc[8];
-    uint32_t cq[4] = {0u, 0u, 0u, 0u};  // Q of the lane's pairs of trajectories
+    uint32_t cq[4] = {0u, 0u, 0u, 0u};  // Q of the lane's pairs of trajectories; MIS: mask of a neighbour in the set
     int neg = 0;
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-    for (int k = 0; k < longest; k += 4) {
-      uint4 p[4];
-      uint32_t sgn[4];
+    for (int k = 0; k < longest; k += kRowDepth) {
+      uint4 p[kRowDepth];
+      uint32_t sgn[kRowDepth];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < kRowDepth; ++q) {
         // past the row's end: zeros, which leave sums and counts as they are
         p[q] = make_uint4(0u, 0u, 0u, 0u);
         sgn[q] = 0u;
@@ -136,13 +143,14 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < kRowDepth; ++q) {
         const uint32_t w[4] = {p[q].x, p[q].y, p[q].z, p[q].w};
         if constexpr (WEIGHTED) neg += sgn[q] & 1u;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const uint32_t m = __hgt2_mask(as2<T2>(w[i]), zero2) ^ sgn[q];
-          cq[i] += m & 0x00010001u;
+          const uint32_t m = __hgt2_mask(as2<T2>(w[i]), thr2) ^ sgn[q];
+          if constexpr (MIS) cq[i] |= m;
+          else cq[i] += m & 0x00010001u;
           X::add(acc[2 * i], acc[2 * i + 1], WEIGHTED ? w[i] ^ (sgn[q] & 0x80008000u) : w[i]);
         }
       }
@@ -156,19 +164,31 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
     uint32_t zw = 0u;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const uint32_t z = __hgt2_mask(as2<T2>(xw[i]), zero2);
-      const uint32_t g0 = cq[i] + ge0, g1 = cq[i] + gt0;
-      zd[i] += z & dn;
-      if (has) zq[i] += z & cq[i];
-      n1[i] += (~(z ^ g0) >> 15) & hb;                     // set and As >= 0, or not set and As < 0
-      n2[i] += (((z & g1) | (~z & ~g0)) >> 15) & hb;       // set and As > 0, or not set and As < 0
+      const uint32_t z = __hgt2_mask(as2<T2>(xw[i]), thr2);
+      if constexpr (MIS) {
+        zd[i] += z & hb;
+        n1[i] += z & cq[i] & hb;
+        n2[i] += ~(z | cq[i]) & hb;
+      } else {
+        const uint32_t g0 = cq[i] + ge0, g1 = cq[i] + gt0;
+        zd[i] += z & dn;
+        if (has) zq[i] += z & cq[i];
+        n1[i] += (~(z ^ g0) >> 15) & hb;                     // set and As >= 0, or not set and As < 0
+        n2[i] += (((z & g1) | (~z & ~g0)) >> 15) & hb;       // set and As > 0, or not set and As < 0
+      }
       float x0, x1, u0, u1;
       X::unpack(xw[i], x0, x1);
       if constexpr (sizeof(TV) == 2) X::unpack(vw[i], u0, u1);
       else u0 = vf[2 * i], u1 = vf[2 * i + 1];
-      // grad = -lambda - 2 acc: doubling is exact, so one rounding either way
       float g0f = acc[2 * i], g1f = acc[2 * i + 1];
-      fma2(g0f, g1f, -2.0f, -a.lambda_);
+      if constexpr (MIS) {
+        mul2(g0f, g1f, a.gamma, a.gamma);
+        g0f = 1.0f - g0f;
+        g1f = 1.0f - g1f;
+      } else {
+        // -lambda - 2 acc: doubling is exact, so one rounding either way
+        fma2(g0f, g1f, -2.0f, -a.lambda_);
+      }
       mul2(g0f, g1f, a.alpha, a.alpha);
       mul2(u0, u1, a.momentum, a.momentum);
       u0 = u0 + g0f;
@@ -192,7 +212,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
         }
       }
       xw[i] = xn;
-      zw |= __hgt2_mask(as2<T2>(xn), zero2) & ((1u << (2 * i)) | (1u << (17 + 2 * i)));
+      zw |= __hgt2_mask(as2<T2>(xn), thr2) & ((1u << (2 * i)) | (1u << (17 + 2 * i)));
     }
     uint32_t word = ((zw | (zw >> 16)) & 0xffu) << (b0 & 31);
     word |= __shfl_xor_sync(0xffffffffu, word, 1);
@@ -212,7 +232,8 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     const int sh = 16 * (e & 1);
-    c0[e] = 2 * ((int)((zd[e >> 1] >> sh) & 0xffffu) - (int)((zq[e >> 1] >> sh) & 0xffffu));
+    c0[e] = (int)((zd[e >> 1] >> sh) & 0xffffu) - (int)((zq[e >> 1] >> sh) & 0xffffu);
+    if constexpr (!MIS) c0[e] *= 2;
     c1[e] = (int)((n1[e >> 1] >> sh) & 0xffffu);
     c2[e] = (int)((n2[e >> 1] >> sh) & 0xffffu);
   }
@@ -222,14 +243,15 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_step_r(StepArgs a, int per) 
 // a row of x takes 4 to 16 lanes; the packed 16-bit sums hold a lane's share of
 // kItemMaxNodes rows of at most 255 entries
 bool step_rows_possible(int B, int x_dtype, int problem, int objective, int max_degree) {
-  return (B == 32 || B == 64 || B == 128) && x_dtype != DT_F32 && problem == PROB_MAXCUT && objective == OBJ_FB &&
-         max_degree <= 255;
+  return (B == 32 || B == 64 || B == 128) && x_dtype != DT_F32 &&
+         (problem == PROB_MIS || (objective == OBJ_FB && max_degree <= 255));
 }
 
 cudaError_t launch_step_rows(const StepArgs& a, int x_dtype, int v_dtype, int sms, cudaStream_t s) {
   StepArgs b = a;
-  // one member graph: four CTAs per SM share its rows; else the items, in parts
-  // until there are as many CTAs
+  // one wave of four CTAs per SM where the rows allow it: one member graph's rows
+  // are shared out, several graphs' items divided (8 and 16 CTAs per SM of fewer
+  // rows: 48 and 57 us against 43, n = 10^5, degree 3, B = 128)
   const int target = 4 * sms;
   int per = 0, grid;
   if (a.g.num_graphs == 1) {
@@ -237,15 +259,16 @@ cudaError_t launch_step_rows(const StepArgs& a, int x_dtype, int v_dtype, int sm
     per = per < 16 ? 16 : (per > kItemMaxNodes ? kItemMaxNodes : per);
     grid = (a.g.n + per - 1) / per;
   } else {
-    b.split = a.g.num_items >= target ? 1 : (target + a.g.num_items - 1) / a.g.num_items;
-    if (b.split > 8) b.split = 8;
+    b.split = target / a.g.num_items;
+    b.split = b.split < 1 ? 1 : (b.split > 8 ? 8 : b.split);
     grid = a.g.num_items * b.split;
   }
   auto go = [&](auto tx, auto tv) -> cudaError_t {
     using TX = decltype(tx);
     using TV = decltype(tv);
-    if (a.g.w) k_step_r<TX, TV, true><<<grid, kRowThreads, 0, s>>>(b, per);
-    else k_step_r<TX, TV, false><<<grid, kRowThreads, 0, s>>>(b, per);
+    if (a.problem == PROB_MIS) k_step_r<TX, TV, true, false><<<grid, kRowThreads, 0, s>>>(b, per);
+    else if (a.g.w) k_step_r<TX, TV, false, true><<<grid, kRowThreads, 0, s>>>(b, per);
+    else k_step_r<TX, TV, false, false><<<grid, kRowThreads, 0, s>>>(b, per);
     return cudaGetLastError();
   };
   if (x_dtype == DT_BF16 && v_dtype == DT_BF16) return go(__nv_bfloat16{}, __nv_bfloat16{});

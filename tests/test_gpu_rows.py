@@ -1,4 +1,4 @@
-"""The row-group step kernel of MaxCut on f_B against the plain global-memory
+"""The row-group step kernel against the plain global-memory
 kernel: the same steps, statistics and bits, at degrees around its batches of
 four neighbours, slices longer than its staged column indices, packed graphs,
 signed weights, and x out of the box or not a number."""
@@ -42,7 +42,7 @@ def both(mq, monkeypatch, G, x0, steps, **kw):
     out = []
     for force in ("rows", "generic"):
         monkeypatch.setenv("MQO_STEP_KERNEL", force)
-        s = mq.Solver(mq.Graph(G), mq.params(problem=1, alpha=0.05, momentum=0.6, lambda_=0.3, **kw))
+        s = mq.Solver(mq.Graph(G), mq.params(alpha=0.05, momentum=0.6, lambda_=0.3, gamma=1.7, **kw))
         assert s.info()["step_kernel"] == ("rows" if force == "rows" else "global")
         s.set_x(x0)
         s.step(steps)
@@ -55,32 +55,34 @@ def both(mq, monkeypatch, G, x0, steps, **kw):
 
 
 @pytest.mark.parametrize("B,xd,vd", [(32, 1, 1), (64, 1, 0), (128, 2, 2), (64, 2, 0), (128, 1, 0)])
-@pytest.mark.parametrize("name", ["regular", "ragged", "long_rows", "packed", "signed", "signed_packed"])
-def test_rows_step_equals_generic(mq, monkeypatch, name, B, xd, vd):
+@pytest.mark.parametrize("problem,name", [(1, n) for n in ("regular", "ragged", "long_rows", "packed", "signed",
+                                                           "signed_packed")]
+                         + [(0, n) for n in ("regular", "ragged", "long_rows", "packed")])
+def test_rows_step_equals_generic(mq, monkeypatch, problem, name, B, xd, vd):
     G = graph(name)
     gen = torch.Generator(device="cuda").manual_seed(B + xd)
-    x0 = ((torch.rand((G.n, B), device="cuda", generator=gen) - 0.5) * 2.6).clamp(-1, 1)
-    both(mq, monkeypatch, G, x0.to(DT[xd]), 4, batch=B, x_dtype=xd, v_dtype=vd)
+    x0 = ((torch.rand((G.n, B), device="cuda", generator=gen) - 0.5) * 2.6).clamp(-problem, 1)
+    both(mq, monkeypatch, G, x0.to(DT[xd]), 4, problem=problem, batch=B, x_dtype=xd, v_dtype=vd)
 
 
-@pytest.mark.parametrize("name", ["ragged", "signed"])
+@pytest.mark.parametrize("problem,name", [(1, "ragged"), (1, "signed"), (0, "ragged")])
 @pytest.mark.parametrize("value", [1e-6, float("nan"), float("inf"), 3.0, -0.0])
-def test_rows_step_irregular_x(mq, monkeypatch, name, value):
+def test_rows_step_irregular_x(mq, monkeypatch, problem, name, value):
     G = graph(name)
     gen = torch.Generator(device="cuda").manual_seed(9)
     x0 = torch.rand((G.n, 32), device="cuda", generator=gen) * 2 - 1
     x0[torch.rand(x0.shape, device="cuda", generator=gen) < 0.02] = value
-    both(mq, monkeypatch, G, x0.to(torch.bfloat16), 1, batch=32, x_dtype=1)
+    both(mq, monkeypatch, G, x0.to(torch.bfloat16), 1, problem=problem, batch=32, x_dtype=1)
 
 
-@pytest.mark.parametrize("name", ["packed", "signed"])
-def test_rows_machine_equals_generic(mq, monkeypatch, name):
+@pytest.mark.parametrize("problem,name", [(0, "packed"), (1, "packed"), (1, "signed")])
+def test_rows_machine_equals_generic(mq, monkeypatch, problem, name):
     """the whole machine: trajectories that do not step keep x and V"""
     G = graph(name)
     out = []
     for force in ("rows", "generic"):
         monkeypatch.setenv("MQO_STEP_KERNEL", force)
-        s = mq.Solver(mq.Graph(G), mq.params(problem=1, batch=32, x_dtype=1, alpha=0.1, momentum=0.5, t_gs=3,
+        s = mq.Solver(mq.Graph(G), mq.params(problem=problem, batch=32, x_dtype=1, alpha=0.1, momentum=0.5, t_gs=3,
                                              descent_cap=20, init_kind=1, sigma=0.1, seed=5))
         s.run(203)
         vals, bits = s.best()
@@ -88,13 +90,18 @@ def test_rows_machine_equals_generic(mq, monkeypatch, name):
     assert out[0] == out[1]
 
 
-def test_rows_step_default(mq):
-    """the default outside shared memory for MaxCut on f_B with 16-bit x; not for the other relaxations, MIS,
-    FP32 x, narrow batches or rows of more than 255 entries"""
-    G = mq.Graph(mi.random_regular(4002, 3, 1))
-    assert mq.Solver(G, mq.params(problem=1, batch=64, x_dtype=1)).info()["step_kernel"] == "rows"
-    for kw in (dict(objective=1), dict(problem=0), dict(x_dtype=0), dict(batch=16)):
-        kw = {**dict(problem=1, batch=64, x_dtype=1), **kw}
-        assert mq.Solver(G, mq.params(**kw)).info()["step_kernel"] != "rows"
+def test_rows_step_default(mq, monkeypatch):
+    """the default with 16-bit x outside shared memory, in shared memory for few member graphs; not for the other
+    relaxations, FP32 x, narrow batches, or a longest row that the rest of the step does not cover"""
+    for name in ("MQO_STEP_KERNEL", "MQO_STEP_ELL", "MQO_COL16"):
+        monkeypatch.delenv(name, raising=False)
+    G = mq.Graph(mi.random_regular(40000, 3, 1))
+    kern = lambda g, **kw: mq.Solver(g, mq.params(**{**dict(problem=1, batch=64, x_dtype=1), **kw})).info()["step_kernel"]
+    assert kern(G) == kern(G, problem=0) == kern(G, x_dtype=2, v_dtype=0) == "rows"
+    for kw in (dict(objective=1), dict(x_dtype=0), dict(batch=16)):
+        assert kern(G, **kw) != "rows"
     hub = mi.from_edges(4002, np.zeros(256, dtype=np.int64), np.arange(1, 257))
-    assert mq.Solver(mq.Graph(hub), mq.params(problem=1, batch=64, x_dtype=1)).info()["step_kernel"] != "rows"
+    assert kern(mq.Graph(hub)) != "rows" and kern(mq.Graph(hub), problem=0) == "staged"
+    assert kern(mq.Graph(mi.erdos_renyi(300, 0.02, 1)), problem=0) == "staged"     # fits in shared memory, two items
+    many = mi.pack([mi.erdos_renyi(100, 0.2, 1)] * 200)
+    assert kern(mq.Graph(many)).startswith("smem")
