@@ -646,12 +646,12 @@ int slice_kb(mqo_solver s) {
 }
 
 // Rows per warp and pitch (bytes between staged rows of x) of the
-// shared-memory step kernel for 2-byte x: 4 trajectories per lane, or 8 with
-// wide lanes; rows of 64 bytes are stored with a 128-byte pitch.
-void ell_shape(int B, bool wide, int* rpw, int* pitch) {
-  const int vec = wide ? 8 : 4;
+// shared-memory step kernel: 2-byte x: 4 trajectories per lane, or 8 with wide
+// lanes; rows of 64 bytes are stored with a 128-byte pitch; float32: 4.
+void ell_shape(int B, int x_dtype, bool wide, int* rpw, int* pitch) {
+  const int vec = wide && x_dtype != DT_F32 ? 8 : 4;
   *rpw = 32 / (B / vec);
-  *pitch = B * 2 == 64 ? 128 : B * 2;
+  *pitch = std::max(B * (int)dtype_size(x_dtype), 128);
 }
 
 // The sliced-ELL arrays for the current batch and lane width, built and
@@ -660,7 +660,7 @@ void ell_shape(int B, bool wide, int* rpw, int* pitch) {
 // to the group's longest row rounded up to 4 entries; vectors on the device.
 mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
   int rpw = 0, pitch = 0;
-  ell_shape(s->S.B, wide, &rpw, &pitch);
+  ell_shape(s->S.B, s->S.p.x_dtype, wide, &rpw, &pitch);
   for (const auto& es : s->ell_sets)
     if (es.rpw == rpw && es.pitch == pitch) return es;
   mqo_solver_s::EllSet es;
@@ -699,7 +699,7 @@ void use_ell(mqo_solver s, bool on) {
   s->step_ell = false;
   s->ell = nullptr;
   s->ell_pos = nullptr;
-  if (!on || !s->ell_ok) return;
+  if (!on || !s->ell_ok || (s->S.p.x_dtype == DT_F32 && !s->S.step_wide)) return;  // float32: 16-byte lanes only
   const mqo_solver_s::EllSet es = ell_set(s, s->S.step_wide != 0);
   if (!es.ok) return;
   s->step_ell = true;
@@ -970,10 +970,10 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     // MQO_STEP_KERNEL=wide: the shared-memory kernel with 16-byte lanes
     s->S.step_wide = force && strcmp(force, "wide") == 0 && step_wide_possible(B, p->x_dtype) ? 1 : 0;
     // the sliced-ELL neighbour stream of the shared-memory kernel where the
-    // layout allows it (2-byte x; MIS: bfloat16 x; MaxCut: no weights);
-    // MQO_STEP_ELL=0: the CSR arrays.
-    s->ell_ok = s->step_smem_max > 0 && p->x_dtype != DT_F32 && (B == 32 || B == 64 || B == 128) &&
-                (p->problem == PROB_MIS ? p->x_dtype == DT_BF16 : g->d_w == nullptr);
+    // layout allows it (MIS: bfloat16 or float32 x; MaxCut: no weights; float32:
+    // B = 32 or 64); MQO_STEP_ELL=0: the CSR arrays.
+    s->ell_ok = s->step_smem_max > 0 && (B == 32 || B == 64 || (B == 128 && p->x_dtype != DT_F32)) &&
+                (p->problem == PROB_MIS ? p->x_dtype != DT_F16 : g->d_w == nullptr);
     // Default: 16-byte lanes with the ELL stream (the fewest instructions
     // per gathered byte).  MQO_STEP_ELL=1: the ELL stream with the lanes
     // MQO_STEP_KERNEL selects (8-byte unless "wide"); MQO_STEP_KERNEL=wide
@@ -1721,7 +1721,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
           if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, c16, 0, 0});
         }
         if (s->ell_ok) {
-          plans.push_back({st, 0, 0, dc, 0, 0, 0, 1, 0});
+          if (S.p.x_dtype != DT_F32) plans.push_back({st, 0, 0, dc, 0, 0, 0, 1, 0});
           if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, 0, 1, 0});
         }
       } else {

@@ -1,6 +1,6 @@
 // mqo_step.cu -- the dispatch of a tick's step to the shared-memory kernel
 // (mqo_step_smem.cuh; here with column indices from the CSR arrays, in
-// mqo_step_ell.cu with the sliced-ELL stream), the tensor-core kernel of dense
+// mqo_step_ell.cu and mqo_step_f32.cu with the sliced-ELL stream), the tensor-core kernel of dense
 // member graphs (mqo_step_dense.cuh), the staged-gather kernel
 // (mqo_step_staged.cu), the row-group kernel (mqo_step_rows.cu) or the
 // global-memory kernel (mqo_step_generic.cu).
@@ -17,6 +17,10 @@ cudaError_t launch_smem_ell(const StepArgs& a, bool wide, size_t smem, bool mis,
 
 // the row-group kernel (mqo_step_rows.cu)
 cudaError_t launch_step_rows(const StepArgs& a, int x_dtype, int v_dtype, int sms, cudaStream_t s);
+
+// the same for float32 x (mqo_step_f32.cu)
+cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const int4* ell, const int2* ell_pos,
+                                int grid, cudaStream_t s);
 
 size_t step_smem_bytes(int B, int x_dtype, int problem, int max_ng) {
   const size_t sx = x_dtype == DT_F32 ? 4 : 2;
@@ -84,6 +88,7 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
   const bool wide = S.step_wide != 0;
   const bool mis = S.p.problem == PROB_MIS;
   const int grid = S.g.num_items;
+  if (ell && xd == DT_F32) return launch_smem_f32_ell(a, smem, mis, ell, ell_pos, grid, stream);
   if (ell) return launch_smem_ell(a, wide, smem, mis, ell, ell_pos, grid, xd, vd, stream);
   if (xd == DT_F32) return launch_tv<float, float>(wide, smem, mis, a, grid, stream);
   if (xd == DT_BF16 && vd == DT_BF16) return launch_tv<__nv_bfloat16, __nv_bfloat16>(wide, smem, mis, a, grid, stream);
