@@ -144,105 +144,135 @@ cudaError_t launch_tick_end(const SolverDev& S, cudaStream_t stream) {
 }
 
 // ---------------------------------------------------------------- apply
-// Each CTA (a slice of one item) first lists, in increasing order, the
-// trajectories of its member graph that have an apply action this tick and
-// caches their actions, reset keys and bases in shared memory; it then visits
-// only those (node, trajectory) pairs, trajectory fastest, so that the x and V
-// writes of one node's listed trajectories are adjacent.  Bit updates are
-// atomic (several listed trajectories share a node's word).
-__global__ void __launch_bounds__(kPairThreads) k_apply(SolverDev S) {
+// Each CTA (a slice of one item) reads the actions of its member graph's
+// trajectories once.  The bit sets then change a word at a time (a node's words
+// belong to one CTA): accepted bits, work sets and the base of a reset by masks
+// of the trajectories with each action.  x, V and the rounding bits are written
+// only for the (node, trajectory) pairs of a reset or an initialisation, listed
+// in increasing order and visited trajectory fastest, so that one node's writes
+// are adjacent.  Bound by latency
+// (chains of small loads, then 2-byte writes to sectors of x and V).  Taking every
+// pair of every action through its own loads and atomics measured 26 us a tick
+// against 21 (512 graphs of about 750 nodes, B = 32); queueing the pairs that need
+// their place in the permutation, so that whole warps compute it, gained nothing.
+__global__ void __launch_bounds__(kPairThreads, 8) k_apply(SolverDev S) {
   __shared__ int s_list[128];
   __shared__ int s_act[128];
   __shared__ uint32_t s_keys[128][6];
   __shared__ int64_t s_rk[128];
   __shared__ int32_t s_o[128];
-  __shared__ int32_t s_pb[128];
+  __shared__ int32_t s_pb[128];   // pool member that is trajectory b's base (< 0: the empty set)
+  __shared__ uint32_t s_mask[4][5];
   __shared__ int s_wcnt[4];
+  __shared__ uint32_t s_base[kItemMaxNodes * 4];
+  // loads that do not depend on one another go out together
   const int64_t t = *S.tick;
-  if (S.any[0] != (int32_t)(t + 1)) return;
+  const int32_t any = S.any[0];
   int it;
   Item item;
-  if (!item_slice(S, it, item)) return;
-  if (S.gflag[item.g] != (int32_t)(t + 1)) return;
+  const bool mine = item_slice(S, it, item);
+  if (any != (int32_t)(t + 1) || !mine) return;
   const int B = S.B, Bw = S.Bw;
   const int g = item.g;
-  // ordered compaction of the acting trajectories (B <= 128: warps 0..3)
+  const int32_t flag = S.gflag[g];
+  const int myact = threadIdx.x < B ? S.act[(int64_t)g * B + threadIdx.x] : 0;
+  if (flag != (int32_t)(t + 1)) return;
+  // masks of the actions, and the trajectories whose x is written, in order
+  // (B <= 128: warps 0..3)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int myact = 0;
-  if (threadIdx.x < B) myact = S.act[(int64_t)g * B + threadIdx.x];
-  const bool on = threadIdx.x < B && (myact & ACT_APPLY_MASK);
-  const unsigned bal = __ballot_sync(0xffffffffu, on);
-  if (warp < 4 && lane == 0) s_wcnt[warp] = __popc(bal);
-  __syncthreads();
-  if (on) {
-    int pos = __popc(bal & ((1u << lane) - 1u));
-    for (int w = 0; w < warp; ++w) pos += s_wcnt[w];
-    const int64_t tau = (int64_t)g * B + threadIdx.x;
-    s_list[pos] = threadIdx.x;
-    s_act[pos] = myact;
-    if (myact & ACT_RESET) {
-      const TrajState& st = S.st[tau];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) s_keys[pos][i] = st.rkeys[i];
-      s_rk[pos] = st.rk;
+  if (warp < 4) {
+    const bool on = myact & (ACT_RESET | ACT_INIT);
+    const unsigned bal = __ballot_sync(0xffffffffu, on);
+    const unsigned zx = __ballot_sync(0xffffffffu, myact & ACT_ACC_ZX);
+    const unsigned wk = __ballot_sync(0xffffffffu, (myact & (ACT_ACC_WORK | ACT_ACC_ZX)) == ACT_ACC_WORK);
+    const unsigned wzx = __ballot_sync(0xffffffffu, myact & ACT_WORK_ZX);
+    const unsigned wb = __ballot_sync(0xffffffffu, (myact & (ACT_WORK_BEST | ACT_WORK_ZX)) == ACT_WORK_BEST);
+    const unsigned pool = __ballot_sync(0xffffffffu, myact & ACT_POOL);
+    if (lane == 0) {
+      s_wcnt[warp] = __popc(bal);
+      s_mask[warp][0] = zx;
+      s_mask[warp][1] = wk;
+      s_mask[warp][2] = wzx;
+      s_mask[warp][3] = wb;
+      s_mask[warp][4] = pool;
     }
-    if (myact & ACT_INIT) s_o[pos] = S.st[tau].o;
-    s_pb[pos] = (myact & ACT_POOL) ? S.pbase[tau] : -1;
+    if (myact & ACT_POOL) s_pb[threadIdx.x] = S.pbase[(int64_t)g * B + threadIdx.x];
+    asm volatile("bar.sync 1, 128;\n" ::: "memory");  // s_wcnt of warps 0..3
+    if (on) {
+      int pos = __popc(bal & ((1u << lane) - 1u));
+      for (int w = 0; w < warp; ++w) pos += s_wcnt[w];
+      const TrajState& st = S.st[(int64_t)g * B + threadIdx.x];
+      s_list[pos] = threadIdx.x;
+      s_act[pos] = myact;
+      if (myact & ACT_RESET) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) s_keys[pos][i] = st.rkeys[i];
+        s_rk[pos] = st.rk;
+      }
+      if (myact & ACT_INIT) s_o[pos] = st.o;
+    }
   }
   __syncthreads();
-  const int nact = s_wcnt[0] + s_wcnt[1] + s_wcnt[2] + s_wcnt[3];
+  const int nset = s_wcnt[0] + s_wcnt[1] + s_wcnt[2] + s_wcnt[3];
   const int nodes = item.v1 - item.v0;
-  const bool mis = S.p.problem == PROB_MIS;
-  const float thr = mis ? 0.5f : 0.0f;
   void* Xc = (t & 1) ? S.X1 : S.X0;
   uint32_t* Zc = (t & 1) ? S.ZX1 : S.ZX0;
   const uint32_t* Zp = (t & 1) ? S.ZX0 : S.ZX1;  // rounding of the x the last step evaluated
+  for (int idx = threadIdx.x; idx < nodes * Bw; idx += blockDim.x) {
+    const int w = idx % Bw;
+    const int64_t i = (int64_t)item.v0 * Bw + idx;
+    const uint32_t zx = s_mask[w][0], wk = s_mask[w][1], wzx = s_mask[w][2], wb = s_mask[w][3];
+    const uint32_t zbest = S.Zbest[i];
+    const uint32_t zp = (zx | wzx) ? Zp[i] : 0u;
+    const uint32_t zwork = (wk | wzx | wb) ? S.Zwork[i] : 0u;
+    const uint32_t zb = (zbest & ~(zx | wk)) | (zp & zx) | (zwork & wk);
+    if (zb != zbest) S.Zbest[i] = zb;
+    // pool mode: the base of a reset / local search is pool member pbase[tau]
+    uint32_t base = zb;
+    if (uint32_t pool = s_mask[w][4]) {
+      base &= ~pool;
+      const uint32_t* member = S.Pool + (i / Bw) * S.Kw;
+      for (; pool; pool &= pool - 1u) {
+        const int b = __ffs(pool) - 1, k = s_pb[32 * w + b];
+        if (k >= 0) base |= ((member[k >> 5] >> (k & 31)) & 1u) << b;
+      }
+    }
+    if (wzx | wb) S.Zwork[i] = (zwork & ~(wzx | wb)) | (zp & wzx) | (base & wb);
+    s_base[idx] = base;
+  }
+  if (nset == 0) return;
+  __syncthreads();
+  const bool mis = S.p.problem == PROB_MIS;
+  const float thr = mis ? 0.5f : 0.0f;
   const int32_t off = S.g.node_off[g];
   const uint32_t n_g = (uint32_t)(S.g.node_off[g + 1] - off);
-  for (int idx = threadIdx.x; idx < nact * nodes; idx += blockDim.x) {
-    const int j = idx % nact;
+  for (int idx = threadIdx.x; idx < nset * nodes; idx += blockDim.x) {
+    const int vi = idx / nset, j = idx - vi * nset;
     const int b = s_list[j];
-    const int64_t v = item.v0 + idx / nact;
-    const int64_t tau = (int64_t)g * B + b;
-    const int act = s_act[j];
-    bool zb = get_bit(S.Zbest, v, Bw, b);
-    if (act & (ACT_ACC_ZX | ACT_ACC_WORK)) {
-      const bool src = (act & ACT_ACC_ZX) ? get_bit(Zp, v, Bw, b) : get_bit(S.Zwork, v, Bw, b);
-      if (src != zb) set_bit_atomic(S.Zbest, v, Bw, b, src);
-      zb = src;
+    const int64_t v = item.v0 + vi;
+    const uint32_t vl = (uint32_t)(v - off);
+    float x;
+    if (s_act[j] & ACT_RESET) {
+      x = reset_x(mis, (s_base[vi * Bw + (b >> 5)] >> (b & 31)) & 1u, n_g, s_keys[j], s_rk[j], vl);
+    } else {
+      x = init_x(S.p, s_o[j], vl, (int64_t)g * B + b, S.g.row_ptr[v + 1] - S.g.row_ptr[v], S.g.dmax[g]);
     }
-    // pool mode: the base of a reset / local search is pool member pbase[tau]
-    bool base = zb;
-    if (act & ACT_POOL) {
-      const int32_t k = s_pb[j];
-      base = k >= 0 && ((S.Pool[v * S.Kw + (k >> 5)] >> (k & 31)) & 1u);
+    const int64_t e = v * B + b;
+    if (S.p.x_dtype == DT_F32) {
+      static_cast<float*>(Xc)[e] = x;
+    } else if (S.p.x_dtype == DT_BF16) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(x);
+      static_cast<__nv_bfloat16*>(Xc)[e] = h;
+      x = __bfloat162float(h);
+    } else {
+      const __half h = __float2half_rn(x);
+      static_cast<__half*>(Xc)[e] = h;
+      x = __half2float(h);
     }
-    if (act & (ACT_WORK_ZX | ACT_WORK_BEST)) {
-      const bool wv = (act & ACT_WORK_ZX) ? get_bit(Zp, v, Bw, b) : base;
-      set_bit_atomic(S.Zwork, v, Bw, b, wv);
-    }
-    if (act & (ACT_RESET | ACT_INIT)) {
-      const uint32_t vl = (uint32_t)(v - off);
-      const int32_t deg = S.g.row_ptr[v + 1] - S.g.row_ptr[v];
-      float x = (act & ACT_RESET) ? reset_x(mis, base, n_g, s_keys[j], s_rk[j], vl)
-                                  : init_x(S.p, s_o[j], vl, tau, deg, S.g.dmax[g]);
-      const int64_t e = v * B + b;
-      if (S.p.x_dtype == DT_F32) {
-        static_cast<float*>(Xc)[e] = x;
-      } else if (S.p.x_dtype == DT_BF16) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(x);
-        static_cast<__nv_bfloat16*>(Xc)[e] = h;
-        x = __bfloat162float(h);
-      } else {
-        const __half h = __float2half_rn(x);
-        static_cast<__half*>(Xc)[e] = h;
-        x = __half2float(h);
-      }
-      if (S.p.v_dtype == DT_F32) static_cast<float*>(S.V)[e] = 0.0f;
-      else if (S.p.v_dtype == DT_BF16) static_cast<__nv_bfloat16*>(S.V)[e] = __float2bfloat16_rn(0.0f);
-      else static_cast<__half*>(S.V)[e] = __float2half_rn(0.0f);
-      set_bit_atomic(Zc, v, Bw, b, x > thr);
-    }
+    if (S.p.v_dtype == DT_F32) static_cast<float*>(S.V)[e] = 0.0f;
+    else if (S.p.v_dtype == DT_BF16) static_cast<__nv_bfloat16*>(S.V)[e] = __float2bfloat16_rn(0.0f);
+    else static_cast<__half*>(S.V)[e] = __float2half_rn(0.0f);
+    set_bit_atomic(Zc, v, Bw, b, x > thr);
   }
 }
 
