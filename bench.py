@@ -92,6 +92,7 @@ AUTOGRAD = dict(desc="f_B autograd: Chung-Lu power law (exponent 2.5, mean degre
                      "forward + backward + projected momentum step", batch=64, lambda_=0.001, lr=0.001, momentum=0.9)
 
 
+SMALL_TICKS = 4096  # ticks per launch of the multi-tick kernel (kSmallTicks in mqo_api.cu)
 MIS_SCALE_NODES = [10_000_000]  # --nodes overrides it (smaller cases for profiling)
 
 
@@ -510,6 +511,8 @@ def measure_solver(mq, G, pkw, xd, vd, steps, warmup, *, autotune=False, clocks_
            "stepped_fraction": float(dsteps.sum()) / float(steps * len(nnz_t)),
            "all_edge_updates": float(G.nnz) * B * steps, "clocks": sampler.summary() if sampler else None,
            "plan": s.info()}
+    if rec["plan"]["small"]:  # one launch, and one that advances the tick, per SMALL_TICKS ticks
+        rec["launches"] = 2 * -(-steps // SMALL_TICKS)
     if tuned:
         rec["plan"]["autotune_ms_per_tick"] = tuned["ms_per_tick"]
     if extra_ticks:
@@ -582,7 +585,32 @@ def oracle_single(G, wl, xd, vd, ticks, objective=0):
 
 
 STEP_KERNEL_NAMES = {"smem": "mqo::k_step_s", "smem_wide": "mqo::k_step_s", "staged": "mqo::k_step_q",
-                     "global": "mqo::k_step_g"}
+                     "global": "mqo::k_step_g", "rows": "mqo::k_step_r"}
+
+
+def step_kernel_name(plan, x_dtype):
+    """The kernel that runs a plan's steps."""
+    if plan.get("small"):
+        return "mqo::k_small (many ticks per launch)"
+    if plan.get("dense"):
+        return "mqo::k_step_t"
+    if x_dtype == "f32" and plan.get("ell"):
+        return "mqo::k_step_f"
+    return STEP_KERNEL_NAMES.get(plan["step_kernel"], plan["step_kernel"])
+
+
+def member_sizes(G):
+    off = getattr(G, "node_offsets", None)
+    return np.diff(off) if off is not None and len(off) > 2 else np.array([G.n])
+
+
+def dense_flops_per_step(G, B):
+    """Tensor-core operations of k_step_t per launch: every member graph's
+    adjacency, rows and columns padded to 128 and 16, times 64 columns (x and
+    its companions) per 32 trajectories."""
+    sizes = member_sizes(G)
+    rows, cols = -(-sizes // 128) * 128, -(-sizes // 16) * 16
+    return float((2.0 * rows * cols).sum()) * 64 * (B // 32)
 
 
 def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak_src, clocks, n_sm, peaks):
@@ -593,13 +621,25 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
     # sliced-ELL stream's 32-bit row offsets (its padding not counted)
     idx = 4 if plan.get("ell") else (2 if plan.get("col16") else 4)
     alg = algorithmic_bytes_per_step(G, B, sx, sv, idx)
+    if plan.get("dense"):  # bit matrices (rows and columns padded to 128) in place of the column indices
+        rows = -(-member_sizes(G) // 128) * 128
+        alg += float((rows.astype(np.int64) ** 2).sum()) / 8 - 4.0 * G.nnz
     achieved = alg / (step_ms / 1e3) / 1e9
     hbm = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
            "algorithmic_bytes_per_launch": alg, "peak_source": peak_src}
     kern = plan["step_kernel"]
-    traffic = step_kernel_traffic(workload, x_dtype, step_variant(plan))
+    variant = step_variant(plan)
+    traffic = None if plan.get("dense") or variant == "rows" or (x_dtype == "f32" and variant.endswith("_ell")) \
+        else step_kernel_traffic(workload, x_dtype, variant)
     gathered = float(G.nnz) * B * sx  # neighbour rows of x read per launch
-    if kern.startswith("smem"):
+    if plan.get("dense"):
+        # the adjacency comes from bit matrices and x once per CTA
+        flops = dense_flops_per_step(G, B)
+        peak = float(peaks.get("bf16_tflops", 1900.0))
+        roof = {"bound": "tensor", "achieved": flops / (step_ms / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
+                "frac": flops / (step_ms / 1e3) / 1e12 / peak, "flops_per_launch": flops, "hbm": hbm,
+                "peak_source": "measured" if "bf16_tflops" in peaks else "fallback"}
+    elif kern.startswith("smem"):
         sm_clock = (clocks or {}).get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))
         derived = 128.0 * n_sm * sm_clock * 1e6 / 1e9
         probe = peaks.get("smem_probe_gbs")
@@ -617,7 +657,7 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
         # is DRAM traffic on top of the algorithmic bytes (measured: traffic)
         roof = dict(hbm, traffic=traffic, gathered_bytes_per_launch=gathered,
                     achieved_incl_gathers=(alg + gathered) / (step_ms / 1e3) / 1e9)
-    roof.update(kernel=STEP_KERNEL_NAMES.get(kern, kern), step_kernel_ms=step_ms, plan=plan)
+    roof.update(kernel=step_kernel_name(plan, x_dtype), step_kernel_ms=step_ms, plan=plan)
     if traffic:
         # DRAM bytes of the committed capture over this launch time, against the same peak
         roof["dram_gbs_from_traffic"] = traffic / (step_ms / 1e3) / 1e9
@@ -1129,8 +1169,8 @@ def app_b_replay(replay):
 
 
 def fb_kernel_bytes(G, B, writes_grad):
-    """col + row_ptr read once, X read once (forward), the gradient written
-    once (backward)."""
+    """col + row_ptr read once, X read once, and where a block of X's size (the
+    gradient, or A X kept for it) is written, that once."""
     return G.nnz * 4 + (G.n + 1) * 4 + G.n * B * 4 + (G.n * B * 4 if writes_grad else 0)
 
 
@@ -1166,7 +1206,7 @@ def _autograd_job(args):
 
 
 def autograd_measure(mq, steps, warmup, *, local, rank, dist, cpu, cpu_target_s=12.0):
-    """The f_B autograd workload: FbObjective forward + fused SpMM backward +
+    """The f_B autograd workload: FbObjective forward (one gather, A X kept) + backward from A X +
     the projected momentum kernel per step; returns its bench record."""
     import torch
     wl = AUTOGRAD
@@ -1220,23 +1260,22 @@ def autograd_measure(mq, steps, warmup, *, local, rank, dist, cpu, cpu_target_s=
     ms_total = e0.elapsed_time(e1)
     eu_step = 2.0 * G.nnz * B
     ms, value = aggregate_ranks(ms_total, eu_step * steps, dist, "cuda")
-    # forward and backward: one launch for rows of <= 512 entries and row
-    # chunks, one more if some row is longer; the momentum step: one
-    per_fb = 1 + int(G.degrees().max() > 512)
-    launches_per_step = 2 * per_fb + 1
-    # the forward launch (f_B per column: one SpMM pass, X read once); the
-    # backward is the same pass plus the gradient write
+    # forward: one launch for rows of <= 512 entries and row chunks, one more if
+    # some row is longer; backward and the momentum step: one each
+    launches_per_step = 1 + int(G.degrees().max() > 512) + 2
+    # the forward (one SpMM pass: X read once, A X written); the backward reads
+    # A X and writes the gradient
     fwd_ms = ph["forward"] / steps
-    alg = fb_kernel_bytes(G, B, False)
+    alg = fb_kernel_bytes(G, B, True)
     peak = float(peaks.get("hbm_gbs", 6800.0))
     achieved = alg / (fwd_ms / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": profile_traffic("fb_kernel_autograd_powerlaw_f32", "fb_seg", ("mqo_grad.cu", "mqo_dev.cuh")),
-            "kernel": "mqo::k_fb_seg (f_B forward pass: the segment-stream kernel plus the long-row chunk "
-                      "kernels; the fused SpMM backward is the same pass plus a write)",
+            "kernel": "mqo::k_fb_seg (f_B forward pass: rows and long-row chunks; the sums of chunks and the "
+                      "objective's memset are in forward_ms too)",
             "algorithmic_bytes_per_launch": alg, "forward_ms": fwd_ms,
             "gathered_bytes_per_launch": float(G.nnz) * B * 4,
-            "backward_hbm_gbs": fb_kernel_bytes(G, B, True) / (ph["backward"] / steps / 1e3) / 1e9,
+            "backward_hbm_gbs": 2.0 * G.n * B * 4 / (ph["backward"] / steps / 1e3) / 1e9,
             "peak_source": "measured" if "hbm_gbs" in peaks else "fallback"}
     # end to end through the public API: X copied from pinned host memory
     # every step, forward + backward + optimiser step, the objective read back
