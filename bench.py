@@ -410,19 +410,27 @@ def source_hash(sources) -> str:
 STEP_SOURCES = {"smem": ("mqo_step.cu", "mqo_step_smem.cuh", "mqo_step.cuh", "mqo_dev.cuh"),
                 "smem_ell": ("mqo_step_ell.cu", "mqo_step_smem.cuh", "mqo_step.cuh", "mqo_dev.cuh"),
                 "global": ("mqo_step_generic.cu", "mqo_step.cuh", "mqo_dev.cuh"),
-                "staged": ("mqo_step_staged.cu", "mqo_step.cuh", "mqo_dev.cuh")}
+                "staged": ("mqo_step_staged.cu", "mqo_step.cuh", "mqo_dev.cuh"),
+                "rows": ("mqo_step_rows.cu", "mqo_x16.cuh", "mqo_step.cuh", "mqo_dev.cuh"),
+                "dense": ("mqo_step_dense.cu", "mqo_step_dense.cuh", "mqo_x16.cuh", "mqo_step.cuh", "mqo_dev.cuh"),
+                "f32_ell": ("mqo_step_f32.cu", "mqo_step.cuh", "mqo_dev.cuh")}
 
 
 def step_variant(plan):
     """Profile variant name of a plan: smem, smem_wide (CSR indices),
-    smem_ell, smem_wide_ell (sliced-ELL stream), staged, global."""
+    smem_ell, smem_wide_ell (sliced-ELL stream), staged, rows, global, dense
+    (tensor cores)."""
+    if plan.get("dense"):
+        return "dense"
     kern = plan["step_kernel"]
     return kern + "_ell" if kern.startswith("smem") and plan.get("ell") else kern
 
 
 def step_kernel_traffic(workload, x_dtype, variant):
     """DRAM bytes per launch of the step kernel variant (step_variant)."""
-    if variant in ("global", "staged"):
+    if x_dtype == "f32" and variant == "smem_wide_ell":
+        variant = "f32_ell"
+    if variant in STEP_SOURCES and not variant.startswith("smem"):
         src = STEP_SOURCES[variant]
     else:
         src = STEP_SOURCES["smem_ell" if variant.endswith("_ell") else "smem"]
@@ -628,16 +636,14 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
     hbm = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
            "algorithmic_bytes_per_launch": alg, "peak_source": peak_src}
     kern = plan["step_kernel"]
-    variant = step_variant(plan)
-    traffic = None if plan.get("dense") or variant == "rows" or (x_dtype == "f32" and variant.endswith("_ell")) \
-        else step_kernel_traffic(workload, x_dtype, variant)
+    traffic = step_kernel_traffic(workload, x_dtype, step_variant(plan))
     gathered = float(G.nnz) * B * sx  # neighbour rows of x read per launch
     if plan.get("dense"):
         # the adjacency comes from bit matrices and x once per CTA
         flops = dense_flops_per_step(G, B)
         peak = float(peaks.get("bf16_tflops", 1900.0))
         roof = {"bound": "tensor", "achieved": flops / (step_ms / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
-                "frac": flops / (step_ms / 1e3) / 1e12 / peak, "flops_per_launch": flops, "hbm": hbm,
+                "frac": flops / (step_ms / 1e3) / 1e12 / peak, "traffic": traffic, "flops_per_launch": flops, "hbm": hbm,
                 "peak_source": "measured" if "bf16_tflops" in peaks else "fallback"}
     elif kern.startswith("smem"):
         sm_clock = (clocks or {}).get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))

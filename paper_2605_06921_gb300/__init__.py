@@ -289,8 +289,9 @@ class Solver:
         return vals, bits
 
     def info(self):
-        """Execution plan: step kernel (smem, smem_wide, staged or global), discrete kernel, trajectories per
-        lane, KB of gathered rows per staged slice, smem bytes, items, counter replicas."""
+        """Execution plan: step kernel (smem, smem_wide, staged, rows or global; dense: the tensor-core kernel instead),
+        small (many ticks per launch), discrete kernel, trajectories per lane, KB of gathered rows per staged slice,
+        smem bytes, items, counter replicas."""
         k, sm, it, r = C.c_int32(), C.c_int64(), C.c_int32(), C.c_int32()
         _check(lib().mqo_solver_info(self.handle, C.byref(k), C.byref(sm), C.byref(it), C.byref(r)))
         return dict(_plan(k.value), smem_bytes=sm.value, items=it.value, replicas=r.value)

@@ -716,7 +716,7 @@ bool serial_tick() {
 
 // the discrete passes fused into one launch
 cudaError_t launch_disc_fused(mqo_solver s, cudaStream_t stream) {
-  if (s->disc_bits) return launch_disc_bits(s->S, s->g->d_bits, s->g->d_bits_off, s->disc_smem, stream);
+  if (s->disc_bits) return launch_disc_bits(s->S, s->g->d_bits, s->g->d_bits_off, s->disc_smem, s->g->sms, stream);
   return launch_disc_graph(s->S, s->disc_smem, stream);
 }
 

@@ -81,16 +81,13 @@ __global__ void __launch_bounds__(kDbThreads) k_disc_bits(SolverDev S, const uin
   __shared__ uint32_t vz[kDbBatch][kDbWords], va[kDbBatch][kDbWords], vf[kDbBatch][kDbWords], vp[kDbBatch][kDbWords];
   __shared__ int s_cnt[32][4];
   __shared__ int s_props[kDbBatch];
-  const int wk = blockIdx.x % S.Bw, g = blockIdx.x / S.Bw;
+  const int parts = gridDim.x / S.g.num_graphs, g = blockIdx.x / parts;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kWarps = kDbThreads / 32;
   const int64_t t = *S.tick;
   if (S.any[1] != (int32_t)(t + 1)) return;
   if (S.gflag[S.g.num_graphs + g] != (int32_t)(t + 1)) return;
   const int B = S.B, Bw = S.Bw;
-  const int myround = S.rnd[(int64_t)g * B + wk * 32 + lane];
-  unsigned active = __ballot_sync(0xffffffffu, myround != RD_NONE);
-  if (!active) return;
   const bool mis = S.p.problem == PROB_MIS;
   const int32_t off = S.g.node_off[g];
   const int n = S.g.node_off[g + 1] - off;
@@ -103,296 +100,302 @@ __global__ void __launch_bounds__(kDbThreads) k_disc_bits(SolverDev S, const uin
   int32_t* gain = owner + kDbBatch * n;                       // [kDbBatch][n] (MaxCut)
   uint32_t* prop = reinterpret_cast<uint32_t*>(gain + (mis ? 0 : kDbBatch * n));  // [kDbBatch][n]: two ends
   uint16_t* propv = reinterpret_cast<uint16_t*>(prop + kDbBatch * n);             // [kDbBatch][n]: proposer
-  for (int v = threadIdx.x; v < n; v += kDbThreads) {
-    const int64_t i = (int64_t)(off + v) * Bw + wk;
-    sW[v] = S.Zwork[i];
-    sA[v] = S.Zaux[i];
-    sF[v] = S.Zfree[i];
-  }
-  for (int i = threadIdx.x; i < 128; i += kDbThreads) s_cnt[i >> 2][i & 3] = 0;
-  __syncthreads();
-
-  while (active) {
-    int b[kDbBatch], rd[kDbBatch];
-    int nb = 0;
-#pragma unroll
-    for (int k = 0; k < kDbBatch; ++k) {
-      b[k] = 0;
-      rd[k] = RD_NONE;
-      if (active) {
-        b[k] = __ffs(active) - 1;
-        rd[k] = __shfl_sync(0xffffffffu, myround, b[k]);
-        active &= active - 1u;
-        nb = k + 1;
-      }
+  for (int wk = blockIdx.x % parts; wk < Bw; wk += parts) {
+    const int myround = S.rnd[(int64_t)g * B + wk * 32 + lane];
+    unsigned active = __ballot_sync(0xffffffffu, myround != RD_NONE);
+    if (!active) continue;
+    for (int v = threadIdx.x; v < n; v += kDbThreads) {
+      const int64_t i = (int64_t)(off + v) * Bw + wk;
+      sW[v] = S.Zwork[i];
+      sA[v] = S.Zaux[i];
+      sF[v] = S.Zfree[i];
     }
-    bool listed = false, rounds = false;
-#pragma unroll
-    for (int k = 0; k < kDbBatch; ++k) {
-      listed |= rd[k] == RD_SWAP || rd[k] == RD_FLIP2;
-      rounds |= rd[k] == RD_DROP || rd[k] == RD_COMPLETE || rd[k] == RD_FLIP1;
-    }
-    // the sets of the batch as bit vectors over the nodes
-    for (int w = warp; w < kDbWords; w += kWarps) {
-      const int v = 32 * w + unperm(lane);
-      const bool in = v < n;
-      const uint32_t xw = in ? sW[v] : 0u, xa = in ? sA[v] : 0u, xf = in ? sF[v] : 0u;
-#pragma unroll
-      for (int k = 0; k < kDbBatch; ++k) {
-        const unsigned mz = __ballot_sync(0xffffffffu, (xw >> b[k]) & 1u);
-        const unsigned ma = __ballot_sync(0xffffffffu, (xa >> b[k]) & 1u);
-        const unsigned mf = __ballot_sync(0xffffffffu, (xf >> b[k]) & 1u);
-        if (lane == 0) vz[k][w] = mz, va[k][w] = ma, vf[k][w] = mf, vp[k][w] = 0u;
-      }
-    }
-    if (threadIdx.x < kDbBatch) s_props[threadIdx.x] = 0;
-    if (listed)
-      for (int v = threadIdx.x; v < n; v += kDbThreads)
-#pragma unroll
-        for (int k = 0; k < kDbBatch; ++k) {
-          owner[k * n + v] = kNoOwner;
-          if (rd[k] == RD_FLIP2) gain[k * n + v] = S.gain[(int64_t)(off + v) * B + wk * 32 + b[k]];
-        }
+    for (int i = threadIdx.x; i < 128; i += kDbThreads) s_cnt[i >> 2][i & 3] = 0;
     __syncthreads();
 
-    // ---------------- pass A: decisions on the snapshot
-    uint32_t change[(2048 + kDbThreads - 1) / kDbThreads];  // per own row: bit k = this row's bit changes
-    if (rounds) {
-      int i = 0;
+    while (active) {
+      int b[kDbBatch], rd[kDbBatch];
+      int nb = 0;
 #pragma unroll
-      for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) change[q] = 0u;
-#pragma unroll
-      for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) {
-        const int v = threadIdx.x + q * kDbThreads;
-        if (v >= n) break;
-        ++i;
-        const int wv = v >> 5;
-        const uint32_t pb = 1u << perm(v & 31), lt = below(v & 31);
-        bool some[kDbBatch];  // some smaller neighbour in the round's set
-#pragma unroll
-        for (int k = 0; k < kDbBatch; ++k) some[k] = false;
-        for (int c = 0; 4 * c <= wv; ++c) {
-          const uint4 r4 = rows.piece(v, c);
-          const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int w = 4 * c + e;
-            const uint32_t m = w < wv ? r[e] : (w == wv ? r[e] & lt : 0u);
-#pragma unroll
-            for (int k = 0; k < kDbBatch; ++k) {
-              const uint32_t* src = rd[k] == RD_DROP ? vz[k] : rd[k] == RD_COMPLETE ? vf[k] : va[k];
-              some[k] |= (m & src[w]) != 0u;
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < kDbBatch; ++k) {
-          bool ch = false;
-          if (rd[k] == RD_DROP) ch = (vz[k][wv] & pb) && some[k];
-          else if (rd[k] == RD_COMPLETE) ch = (vf[k][wv] & pb) && !some[k];
-          else if (rd[k] == RD_FLIP1) ch = (va[k][wv] & pb) && !some[k];
-          change[q] |= (uint32_t)ch << k;
+      for (int k = 0; k < kDbBatch; ++k) {
+        b[k] = 0;
+        rd[k] = RD_NONE;
+        if (active) {
+          b[k] = __ffs(active) - 1;
+          rd[k] = __shfl_sync(0xffffffffu, myround, b[k]);
+          active &= active - 1u;
+          nb = k + 1;
         }
       }
-    }
+      bool listed = false, rounds = false;
 #pragma unroll
-    for (int k = 0; k < kDbBatch; ++k) {
-      if (rd[k] == RD_SWAP) {
-        // a warp per set node v: the first pair (in CSR order of N(v)) of
-        // non-adjacent tight neighbours
-        int task = 0;
-        for (int w = 0; w < words; ++w) {
-          uint32_t m = vz[k][w];
-          while (m) {
-            const int v = 32 * w + unperm(__ffs(m) - 1);
-            m &= m - 1u;
-            if (task++ % kWarps != warp) continue;
-            uint32_t r0 = lane < words ? natural(rows.word(v, lane) & va[k][lane]) : 0u;
-            uint32_t r1 = 32 + lane < words ? natural(rows.word(v, 32 + lane) & va[k][32 + lane]) : 0u;
-            int fa, fb = -1;
-            while ((fa = warp_first(r0, r1)) >= 0) {
-              if ((fa >> 5) == lane) r0 &= r0 - 1u;
-              if ((fa >> 5) == 32 + lane) r1 &= r1 - 1u;
-              const uint32_t n0 = lane < words ? r0 & ~natural(rows.word(fa, lane)) : 0u;
-              const uint32_t n1 = 32 + lane < words ? r1 & ~natural(rows.word(fa, 32 + lane)) : 0u;
-              fb = warp_first(n0, n1);
-              if (fb >= 0) break;
-            }
-            if (fb >= 0 && lane == 0) {
-              owner[k * n + fa] = v;
-              owner[k * n + fb] = v;
-              atomicOr(&vp[k][fa >> 5], 1u << perm(fa & 31));
-              atomicOr(&vp[k][fb >> 5], 1u << perm(fb & 31));
-              const int i = atomicAdd(&s_props[k], 1);
-              prop[k * n + i] = (uint32_t)fa | ((uint32_t)fb << 16);
-              propv[k * n + i] = (uint16_t)v;
-            }
-          }
+      for (int k = 0; k < kDbBatch; ++k) {
+        listed |= rd[k] == RD_SWAP || rd[k] == RD_FLIP2;
+        rounds |= rd[k] == RD_DROP || rd[k] == RD_COMPLETE || rd[k] == RD_FLIP1;
+      }
+      // the sets of the batch as bit vectors over the nodes
+      for (int w = warp; w < kDbWords; w += kWarps) {
+        const int v = 32 * w + unperm(lane);
+        const bool in = v < n;
+        const uint32_t xw = in ? sW[v] : 0u, xa = in ? sA[v] : 0u, xf = in ? sF[v] : 0u;
+#pragma unroll
+        for (int k = 0; k < kDbBatch; ++k) {
+          const unsigned mz = __ballot_sync(0xffffffffu, (xw >> b[k]) & 1u);
+          const unsigned ma = __ballot_sync(0xffffffffu, (xa >> b[k]) & 1u);
+          const unsigned mf = __ballot_sync(0xffffffffu, (xf >> b[k]) & 1u);
+          if (lane == 0) vz[k][w] = mz, va[k][w] = ma, vf[k][w] = mf, vp[k][w] = 0u;
         }
-      } else if (rd[k] == RD_FLIP2) {
-        // node v proposes its first neighbour u > v on the other side with a
-        // positive pair gain
-        for (int v = threadIdx.x; v < n; v += kDbThreads) {
+      }
+      if (threadIdx.x < kDbBatch) s_props[threadIdx.x] = 0;
+      if (listed)
+        for (int v = threadIdx.x; v < n; v += kDbThreads)
+#pragma unroll
+          for (int k = 0; k < kDbBatch; ++k) {
+            owner[k * n + v] = kNoOwner;
+            if (rd[k] == RD_FLIP2) gain[k * n + v] = S.gain[(int64_t)(off + v) * B + wk * 32 + b[k]];
+          }
+      __syncthreads();
+
+      // ---------------- pass A: decisions on the snapshot
+      uint32_t change[(2048 + kDbThreads - 1) / kDbThreads];  // per own row: bit k = this row's bit changes
+      if (rounds) {
+        int i = 0;
+#pragma unroll
+        for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) change[q] = 0u;
+#pragma unroll
+        for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) {
+          const int v = threadIdx.x + q * kDbThreads;
+          if (v >= n) break;
+          ++i;
           const int wv = v >> 5;
-          const bool zv = (vz[k][wv] >> perm(v & 31)) & 1u;
-          const int ga = gain[k * n + v];
-          int fu = -1;
-          for (int c = wv >> 2; c < rows.nc && fu < 0; ++c) {
+          const uint32_t pb = 1u << perm(v & 31), lt = below(v & 31);
+          bool some[kDbBatch];  // some smaller neighbour in the round's set
+#pragma unroll
+          for (int k = 0; k < kDbBatch; ++k) some[k] = false;
+          for (int c = 0; 4 * c <= wv; ++c) {
             const uint4 r4 = rows.piece(v, c);
             const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int w = 4 * c + e;
-              if (w < wv || fu >= 0) continue;
-              uint32_t m = r[e] & (zv ? ~vz[k][w] : vz[k][w]);
-              if (w == wv) m &= ~(below(v & 31) | (1u << perm(v & 31)));
-              m = natural(m);
-              while (m) {
-                const int u = 32 * w + __ffs(m) - 1;
-                m &= m - 1u;
-                if (ga + gain[k * n + u] + 2 > 0) {
-                  fu = u;
-                  break;
-                }
+              const uint32_t m = w < wv ? r[e] : (w == wv ? r[e] & lt : 0u);
+#pragma unroll
+              for (int k = 0; k < kDbBatch; ++k) {
+                const uint32_t* src = rd[k] == RD_DROP ? vz[k] : rd[k] == RD_COMPLETE ? vf[k] : va[k];
+                some[k] |= (m & src[w]) != 0u;
               }
             }
           }
-          if (fu >= 0) {
-            atomicMin(&owner[k * n + v], v);
-            atomicMin(&owner[k * n + fu], v);
-            atomicOr(&vp[k][wv], 1u << perm(v & 31));
-            atomicOr(&vp[k][fu >> 5], 1u << perm(fu & 31));
-            const int i = atomicAdd(&s_props[k], 1);
-            prop[k * n + i] = (uint32_t)v | ((uint32_t)fu << 16);
-            propv[k * n + i] = (uint16_t)v;
+#pragma unroll
+          for (int k = 0; k < kDbBatch; ++k) {
+            bool ch = false;
+            if (rd[k] == RD_DROP) ch = (vz[k][wv] & pb) && some[k];
+            else if (rd[k] == RD_COMPLETE) ch = (vf[k][wv] & pb) && !some[k];
+            else if (rd[k] == RD_FLIP1) ch = (va[k][wv] & pb) && !some[k];
+            change[q] |= (uint32_t)ch << k;
           }
         }
       }
-    }
-    __syncthreads();
-
-    // ---------------- pass B: commits
-    if (rounds) {
-#pragma unroll
-      for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) {
-        const int v = threadIdx.x + q * kDbThreads;
-        if (v >= n) break;
-#pragma unroll
-        for (int k = 0; k < kDbBatch; ++k)
-          if ((change[q] >> k) & 1u) {
-            atomicXor(&vz[k][v >> 5], 1u << perm(v & 31));  // drops clear, completions set, flips toggle
-            atomicAdd(&s_cnt[b[k]][3], 1);
-          }
-      }
-    }
-    if (listed) {
 #pragma unroll
       for (int k = 0; k < kDbBatch; ++k) {
-        const bool flip2 = rd[k] == RD_FLIP2;
-        if (rd[k] != RD_SWAP && !flip2) continue;
-        // a proposal commits if no neighbour of its two ends (other than the
-        // ends) is claimed by a smaller proposer; a 2-flip also has to hold
-        // both its claims
-        for (int i = warp; i < s_props[k]; i += kWarps) {
-          const int v = propv[k * n + i];
-          const int e0 = (int)(prop[k * n + i] & 0xffffu), e1 = (int)(prop[k * n + i] >> 16);
-          bool bad = flip2 && (owner[k * n + e0] != v || owner[k * n + e1] != v);
-          for (int w = lane; w < words; w += 32) {
-            uint32_t m = (rows.word(e0, w) | rows.word(e1, w)) & vp[k][w];
+        if (rd[k] == RD_SWAP) {
+          // a warp per set node v: the first pair (in CSR order of N(v)) of
+          // non-adjacent tight neighbours
+          int task = 0;
+          for (int w = 0; w < words; ++w) {
+            uint32_t m = vz[k][w];
             while (m) {
-              const int u = 32 * w + unperm(__ffs(m) - 1);
+              const int v = 32 * w + unperm(__ffs(m) - 1);
               m &= m - 1u;
-              if (u != e0 && u != e1) bad |= owner[k * n + u] < v;
+              if (task++ % kWarps != warp) continue;
+              uint32_t r0 = lane < words ? natural(rows.word(v, lane) & va[k][lane]) : 0u;
+              uint32_t r1 = 32 + lane < words ? natural(rows.word(v, 32 + lane) & va[k][32 + lane]) : 0u;
+              int fa, fb = -1;
+              while ((fa = warp_first(r0, r1)) >= 0) {
+                if ((fa >> 5) == lane) r0 &= r0 - 1u;
+                if ((fa >> 5) == 32 + lane) r1 &= r1 - 1u;
+                const uint32_t n0 = lane < words ? r0 & ~natural(rows.word(fa, lane)) : 0u;
+                const uint32_t n1 = 32 + lane < words ? r1 & ~natural(rows.word(fa, 32 + lane)) : 0u;
+                fb = warp_first(n0, n1);
+                if (fb >= 0) break;
+              }
+              if (fb >= 0 && lane == 0) {
+                owner[k * n + fa] = v;
+                owner[k * n + fb] = v;
+                atomicOr(&vp[k][fa >> 5], 1u << perm(fa & 31));
+                atomicOr(&vp[k][fb >> 5], 1u << perm(fb & 31));
+                const int i = atomicAdd(&s_props[k], 1);
+                prop[k * n + i] = (uint32_t)fa | ((uint32_t)fb << 16);
+                propv[k * n + i] = (uint16_t)v;
+              }
             }
           }
-          if (!__any_sync(0xffffffffu, bad) && lane == 0) {
-            if (!flip2) atomicXor(&vz[k][v >> 5], 1u << perm(v & 31));
-            atomicXor(&vz[k][e0 >> 5], 1u << perm(e0 & 31));
-            atomicXor(&vz[k][e1 >> 5], 1u << perm(e1 & 31));
-            atomicAdd(&s_cnt[b[k]][3], 1);
+        } else if (rd[k] == RD_FLIP2) {
+          // node v proposes its first neighbour u > v on the other side with a
+          // positive pair gain
+          for (int v = threadIdx.x; v < n; v += kDbThreads) {
+            const int wv = v >> 5;
+            const bool zv = (vz[k][wv] >> perm(v & 31)) & 1u;
+            const int ga = gain[k * n + v];
+            int fu = -1;
+            for (int c = wv >> 2; c < rows.nc && fu < 0; ++c) {
+              const uint4 r4 = rows.piece(v, c);
+              const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const int w = 4 * c + e;
+                if (w < wv || fu >= 0) continue;
+                uint32_t m = r[e] & (zv ? ~vz[k][w] : vz[k][w]);
+                if (w == wv) m &= ~(below(v & 31) | (1u << perm(v & 31)));
+                m = natural(m);
+                while (m) {
+                  const int u = 32 * w + __ffs(m) - 1;
+                  m &= m - 1u;
+                  if (ga + gain[k * n + u] + 2 > 0) {
+                    fu = u;
+                    break;
+                  }
+                }
+              }
+            }
+            if (fu >= 0) {
+              atomicMin(&owner[k * n + v], v);
+              atomicMin(&owner[k * n + fu], v);
+              atomicOr(&vp[k][wv], 1u << perm(v & 31));
+              atomicOr(&vp[k][fu >> 5], 1u << perm(fu & 31));
+              const int i = atomicAdd(&s_props[k], 1);
+              prop[k * n + i] = (uint32_t)v | ((uint32_t)fu << 16);
+              propv[k * n + i] = (uint16_t)v;
+            }
           }
         }
       }
-    }
-    __syncthreads();
+      __syncthreads();
 
-    // ---------------- pass C: counts of the (new) work sets
-    int acc[kDbBatch][3];
+      // ---------------- pass B: commits
+      if (rounds) {
 #pragma unroll
-    for (int k = 0; k < kDbBatch; ++k) acc[k][0] = acc[k][1] = acc[k][2] = 0;
-    for (int v = threadIdx.x; v < n; v += kDbThreads) {
-      int cnt[kDbBatch], deg = 0;
+        for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) {
+          const int v = threadIdx.x + q * kDbThreads;
+          if (v >= n) break;
 #pragma unroll
-      for (int k = 0; k < kDbBatch; ++k) cnt[k] = 0;
-#pragma unroll 4
-      for (int c = 0; c < rows.nc; ++c) {
-        const uint4 r4 = rows.piece(v, c);
-        const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (!mis) deg += __popc(r[e]);
-#pragma unroll
-          for (int k = 0; k < kDbBatch; ++k) cnt[k] += __popc(r[e] & vz[k][4 * c + e]);
+          for (int k = 0; k < kDbBatch; ++k)
+            if ((change[q] >> k) & 1u) {
+              atomicXor(&vz[k][v >> 5], 1u << perm(v & 31));  // drops clear, completions set, flips toggle
+              atomicAdd(&s_cnt[b[k]][3], 1);
+            }
         }
       }
-      uint32_t xw = sW[v], xa = sA[v], xf = sF[v];
+      if (listed) {
+#pragma unroll
+        for (int k = 0; k < kDbBatch; ++k) {
+          const bool flip2 = rd[k] == RD_FLIP2;
+          if (rd[k] != RD_SWAP && !flip2) continue;
+          // a proposal commits if no neighbour of its two ends (other than the
+          // ends) is claimed by a smaller proposer; a 2-flip also has to hold
+          // both its claims
+          for (int i = warp; i < s_props[k]; i += kWarps) {
+            const int v = propv[k * n + i];
+            const int e0 = (int)(prop[k * n + i] & 0xffffu), e1 = (int)(prop[k * n + i] >> 16);
+            bool bad = flip2 && (owner[k * n + e0] != v || owner[k * n + e1] != v);
+            for (int w = lane; w < words; w += 32) {
+              uint32_t m = (rows.word(e0, w) | rows.word(e1, w)) & vp[k][w];
+              while (m) {
+                const int u = 32 * w + unperm(__ffs(m) - 1);
+                m &= m - 1u;
+                if (u != e0 && u != e1) bad |= owner[k * n + u] < v;
+              }
+            }
+            if (!__any_sync(0xffffffffu, bad) && lane == 0) {
+              if (!flip2) atomicXor(&vz[k][v >> 5], 1u << perm(v & 31));
+              atomicXor(&vz[k][e0 >> 5], 1u << perm(e0 & 31));
+              atomicXor(&vz[k][e1 >> 5], 1u << perm(e1 & 31));
+              atomicAdd(&s_cnt[b[k]][3], 1);
+            }
+          }
+        }
+      }
+      __syncthreads();
+
+      // ---------------- pass C: counts of the (new) work sets
+      int acc[kDbBatch][3];
+#pragma unroll
+      for (int k = 0; k < kDbBatch; ++k) acc[k][0] = acc[k][1] = acc[k][2] = 0;
+      for (int v = threadIdx.x; v < n; v += kDbThreads) {
+        int cnt[kDbBatch], deg = 0;
+#pragma unroll
+        for (int k = 0; k < kDbBatch; ++k) cnt[k] = 0;
+#pragma unroll 4
+        for (int c = 0; c < rows.nc; ++c) {
+          const uint4 r4 = rows.piece(v, c);
+          const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (!mis) deg += __popc(r[e]);
+#pragma unroll
+            for (int k = 0; k < kDbBatch; ++k) cnt[k] += __popc(r[e] & vz[k][4 * c + e]);
+          }
+        }
+        uint32_t xw = sW[v], xa = sA[v], xf = sF[v];
+#pragma unroll
+        for (int k = 0; k < kDbBatch; ++k) {
+          if (k >= nb) break;
+          const uint32_t bit = 1u << b[k];
+          const bool z = (vz[k][v >> 5] >> perm(v & 31)) & 1u;
+          bool aux, fr = false;
+          if (mis) {
+            const bool one = cnt[k] >= 1;
+            acc[k][0] += z;
+            acc[k][1] += z && one;
+            fr = !z && !one;
+            acc[k][2] += fr;
+            aux = !z && cnt[k] == 1;  // tight: exactly one neighbour in the set
+            xf = fr ? xf | bit : xf & ~bit;
+          } else {
+            const int as = 2 * cnt[k] - deg;
+            acc[k][0] += z ? deg - cnt[k] : cnt[k];
+            acc[k][1] += !(z ? as <= -1 : as >= 0);  // f_B rule (Thm 3.6), any objective
+            const int gn = z ? as : -as;
+            aux = gn > 0;
+            acc[k][2] += aux;
+            S.gain[(int64_t)(off + v) * B + wk * 32 + b[k]] = gn;
+          }
+          S.owner[(int64_t)(off + v) * B + wk * 32 + b[k]] = kNoOwner;  // as the list kernels leave it
+          xw = z ? xw | bit : xw & ~bit;
+          xa = aux ? xa | bit : xa & ~bit;
+        }
+        sW[v] = xw;
+        sA[v] = xa;
+        sF[v] = xf;
+      }
 #pragma unroll
       for (int k = 0; k < kDbBatch; ++k) {
         if (k >= nb) break;
-        const uint32_t bit = 1u << b[k];
-        const bool z = (vz[k][v >> 5] >> perm(v & 31)) & 1u;
-        bool aux, fr = false;
-        if (mis) {
-          const bool one = cnt[k] >= 1;
-          acc[k][0] += z;
-          acc[k][1] += z && one;
-          fr = !z && !one;
-          acc[k][2] += fr;
-          aux = !z && cnt[k] == 1;  // tight: exactly one neighbour in the set
-          xf = fr ? xf | bit : xf & ~bit;
-        } else {
-          const int as = 2 * cnt[k] - deg;
-          acc[k][0] += z ? deg - cnt[k] : cnt[k];
-          acc[k][1] += !(z ? as <= -1 : as >= 0);  // f_B rule (Thm 3.6), any objective
-          const int gn = z ? as : -as;
-          aux = gn > 0;
-          acc[k][2] += aux;
-          S.gain[(int64_t)(off + v) * B + wk * 32 + b[k]] = gn;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const int sum = __reduce_add_sync(0xffffffffu, acc[k][i]);
+          if (lane == 0 && sum) atomicAdd(&s_cnt[b[k]][i], sum);
         }
-        S.owner[(int64_t)(off + v) * B + wk * 32 + b[k]] = kNoOwner;  // as the list kernels leave it
-        xw = z ? xw | bit : xw & ~bit;
-        xa = aux ? xa | bit : xa & ~bit;
       }
-      sW[v] = xw;
-      sA[v] = xa;
-      sF[v] = xf;
+      __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < kDbBatch; ++k) {
-      if (k >= nb) break;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int sum = __reduce_add_sync(0xffffffffu, acc[k][i]);
-        if (lane == 0 && sum) atomicAdd(&s_cnt[b[k]][i], sum);
-      }
-    }
-    __syncthreads();
-  }
 
-  for (int v = threadIdx.x; v < n; v += kDbThreads) {
-    const int64_t i = (int64_t)(off + v) * Bw + wk;
-    S.Zwork[i] = sW[v];
-    S.Zaux[i] = sA[v];
-    S.Zfree[i] = sF[v];
-  }
-  if (threadIdx.x < 128) {
-    const int tb = threadIdx.x >> 2, k = threadIdx.x & 3;
-    const int val = s_cnt[tb][k];
-    if (val) {
-      Counters* c = S.cnt + ((int64_t)g * B + wk * 32 + tb) * S.R;  // replica 0
-      unsigned long long* p = k == 0 ? &c->value : k == 1 ? &c->a : k == 2 ? &c->b : &c->commits;
-      atomicAdd(p, (unsigned long long)(long long)val);
+    for (int v = threadIdx.x; v < n; v += kDbThreads) {
+      const int64_t i = (int64_t)(off + v) * Bw + wk;
+      S.Zwork[i] = sW[v];
+      S.Zaux[i] = sA[v];
+      S.Zfree[i] = sF[v];
     }
+    if (threadIdx.x < 128) {
+      const int tb = threadIdx.x >> 2, k = threadIdx.x & 3;
+      const int val = s_cnt[tb][k];
+      if (val) {
+        Counters* c = S.cnt + ((int64_t)g * B + wk * 32 + tb) * S.R;  // replica 0
+        unsigned long long* p = k == 0 ? &c->value : k == 1 ? &c->a : k == 2 ? &c->b : &c->commits;
+        atomicAdd(p, (unsigned long long)(long long)val);
+      }
+    }
+    __syncthreads();  // before the next word's sets
   }
 }
 
@@ -493,10 +496,16 @@ size_t disc_bits_smem_bytes(int problem, int max_ng) {
 }
 
 cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, size_t smem,
-                             cudaStream_t stream) {
+                             int sms, cudaStream_t stream) {
+  // a CTA per member graph and word of trajectories while there are SMs for
+  // them, else a CTA takes several words (one CTA fits on an SM, and a tick
+  // without rounds pays for the launch of each: 407 graphs, B = 128: 9.8 us with
+  // a CTA per word, 7.3 with one per graph)
+  int parts = S.Bw;
+  while (parts > 1 && S.g.num_graphs * parts > sms) parts /= 2;
   cudaError_t e = cudaFuncSetAttribute(k_disc_bits, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_disc_bits<<<S.g.num_graphs * S.Bw, kDbThreads, smem, stream>>>(S, bits, bits_off);
+  k_disc_bits<<<S.g.num_graphs * parts, kDbThreads, smem, stream>>>(S, bits, bits_off);
   return cudaGetLastError();
 }
 

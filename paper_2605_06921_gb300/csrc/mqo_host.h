@@ -57,7 +57,7 @@ cudaError_t launch_disc_graph(const SolverDev& S, size_t smem, cudaStream_t stre
 // the same for member graphs with bit matrices (mqo_disc_bits.cu)
 size_t disc_bits_smem_bytes(int problem, int max_ng);
 cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, size_t smem,
-                             cudaStream_t stream);
+                             int sms, cudaStream_t stream);
 cudaError_t launch_tick_end(const SolverDev& S, cudaStream_t stream);
 cudaError_t launch_round_bits(const SolverDev& S, uint32_t* z, cudaStream_t stream);
 cudaError_t launch_eval(const SolverDev& S, const uint32_t* z, Counters* out, cudaStream_t stream);

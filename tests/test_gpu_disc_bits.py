@@ -21,7 +21,7 @@ def mq():
 
 @pytest.mark.parametrize("problem", [0, 1])
 @pytest.mark.parametrize("B,xd", [(32, 1), (64, 0), (128, 1)])
-@pytest.mark.parametrize("sizes,p", [((40, 64, 33), 0.45), ((128, 129, 200), 0.2), ((600,), 0.08)])
+@pytest.mark.parametrize("sizes,p", [((40, 64, 33), 0.45), ((128, 129, 200), 0.2), ((600,), 0.08), ((40,) * 160, 0.3)])
 def test_bits_equal_lists(mq, monkeypatch, problem, B, xd, sizes, p):
     gs = [mi.erdos_renyi(n, p, n) for n in sizes]
     G = mi.pack(gs) if len(gs) > 1 else gs[0]
