@@ -55,7 +55,7 @@ typedef enum {
   MQO_EGRAPH = -2,  /* CSR failed validation (see mqo_last_error) */
   MQO_ENOMEM = -3,  /* device or host allocation failed */
   MQO_ECUDA = -4,   /* a CUDA call failed; the solver is poisoned */
-  MQO_ETIMEOUT = -5,/* reserved: no entry point waits on the device */
+  MQO_ETIMEOUT = -5,/* a bounded wait inside a step kernel ran out (reported by mqo_best and mqo_traj_state) */
   MQO_ESTATE = -6   /* solver poisoned by an earlier failure */
 } mqo_status;
 
@@ -305,8 +305,13 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * per entry of device memory), bit 17 = the shared-memory step kernel reads
  * its neighbours from the solver's sliced-ELL stream (the rows of a warp
  * padded to a common length, four neighbour offsets per 16-byte vector;
- * 2-byte x, MIS with bfloat16 x or unweighted MaxCut; about 4 bytes of
- * device memory per entry and lane width); *smem_bytes = the
+ * MIS with bfloat16 or float32 x, or unweighted MaxCut; about 4 bytes of
+ * device memory per entry and lane width), bit 18 = the tensor-core kernel
+ * of dense member graphs (bit 0 is set too: it keeps x in shared memory),
+ * bit 19 = mqo_run and mqo_step take many ticks per launch, one CTA per
+ * member graph (small graphs; the other bits describe the plan of single
+ * ticks, which mqo_run_timed takes), bit 20 = the row-group kernel (16-bit x,
+ * neighbour rows read from L2, bits 0 and 3 clear); *smem_bytes = the
  * shared-memory step kernel's dynamic shared memory per CTA; *items = work
  * items (node ranges of at most 256 nodes); *replicas = counter replicas per
  * trajectory.
@@ -315,10 +320,11 @@ MQO_API mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* 
                                    int32_t* replicas);
 
 /*
- * Autotuner of the launch plan: every plan the solver can run (shared-memory
- * or global-memory step kernel; for the former lane width and neighbour
- * stream, for the latter each choice of trajectories per lane, i.e. lanes
- * per row, and of staged slices; fused or node-parallel discrete passes)
+ * Autotuner of the launch plan: every plan the solver can run (shared-memory,
+ * tensor-core, row-group or global-memory step kernel; for the first lane
+ * width and neighbour stream, for the last each choice of trajectories per
+ * lane, i.e. lanes per row, and of staged slices; fused or node-parallel
+ * discrete passes; many ticks per launch)
  * runs `ticks` machine ticks from the current state; the state is restored
  * after every trial, so tuning changes no result (all plans compute the same
  * ticks bit for bit).  The current plan is timed first; another replaces it
