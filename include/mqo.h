@@ -305,8 +305,9 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * per entry of device memory), bit 17 = the shared-memory step kernel reads
  * its neighbours from the solver's sliced-ELL stream (the rows of a warp
  * padded to a common length, four neighbour offsets per 16-byte vector;
- * MIS with bfloat16 or float32 x, or unweighted MaxCut; about 4 bytes of
- * device memory per entry and lane width), bit 18 = the tensor-core kernel
+ * MIS with bfloat16 or float32 x, or unweighted MaxCut; every type for 4 to
+ * 16 trajectories, whose x it stages as float32; about 4 bytes of device
+ * memory per entry and lane width), bit 18 = the tensor-core kernel
  * of dense member graphs (bit 0 is set too: it keeps x in shared memory),
  * bit 19 = mqo_run and mqo_step take many ticks per launch, one CTA per
  * member graph (small graphs; the other bits describe the plan of single

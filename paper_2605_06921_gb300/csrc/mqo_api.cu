@@ -153,6 +153,7 @@ struct mqo_solver_s {
   };
   std::vector<EllSet> ell_sets;
   bool ell_ok = false;           // the layout allows the ELL stream
+  bool ell_only = false;         // the shared-memory kernel needs it (B < 32)
   bool step_ell = false;         // the current plan uses it
   const int4* ell = nullptr;     // its arrays for the current lane width
   const int2* ell_pos = nullptr;
@@ -647,11 +648,12 @@ int slice_kb(mqo_solver s) {
 
 // Rows per warp and pitch (bytes between staged rows of x) of the
 // shared-memory step kernel: 2-byte x: 4 trajectories per lane, or 8 with wide
-// lanes; rows of 64 bytes are stored with a 128-byte pitch; float32: 4.
+// lanes; rows of 64 bytes are stored with a 128-byte pitch; float32, and every type
+// below 32 trajectories: 4, staged as float32.
 void ell_shape(int B, int x_dtype, bool wide, int* rpw, int* pitch) {
-  const int vec = wide && x_dtype != DT_F32 ? 8 : 4;
+  const int vec = wide && x_dtype != DT_F32 && B >= 32 ? 8 : 4;
   *rpw = 32 / (B / vec);
-  *pitch = std::max(B * (int)dtype_size(x_dtype), 128);
+  *pitch = x_dtype == DT_F32 || B < 32 ? B * 4 : std::max(B * 2, 128);
 }
 
 // The sliced-ELL arrays for the current batch and lane width, built and
@@ -950,8 +952,10 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     const char* force = getenv("MQO_STEP_KERNEL");
     const bool generic = force && strcmp(force, "generic") == 0;
     const bool staged = force && strcmp(force, "staged") == 0;
-    s->step_smem_max = (B >= 32 && need <= kStepSmemLimit) ? need : 0;
-    s->step_smem = (generic || staged) ? 0 : s->step_smem_max;
+    const bool ell_plain = p->problem == PROB_MIS || g->d_w == nullptr;
+    s->ell_only = (B == 4 || B == 8 || B == 16) && ell_plain;
+    s->step_smem_max = ((B >= 32 || s->ell_only) && need <= kStepSmemLimit) ? need : 0;
+    s->step_smem = (generic || staged || (s->ell_only && force)) ? 0 : s->step_smem_max;
     if (staged_possible(B, p->x_dtype, p->v_dtype)) {
       // the smallest slice capacity from the default up that holds every row
       for (int kb = kDefaultSliceKB; kb <= 128 && !s->staged_ok; kb *= 2) {
@@ -971,9 +975,11 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     s->S.step_wide = force && strcmp(force, "wide") == 0 && step_wide_possible(B, p->x_dtype) ? 1 : 0;
     // the sliced-ELL neighbour stream of the shared-memory kernel where the
     // layout allows it (MIS: bfloat16 or float32 x; MaxCut: no weights; float32:
-    // B = 32 or 64); MQO_STEP_ELL=0: the CSR arrays.
-    s->ell_ok = s->step_smem_max > 0 && (B == 32 || B == 64 || (B == 128 && p->x_dtype != DT_F32)) &&
-                (p->problem == PROB_MIS ? p->x_dtype != DT_F16 : g->d_w == nullptr);
+    // B <= 64, from B = 4, where below 32 there is no CSR form); MQO_STEP_ELL=0: the
+    // CSR arrays.
+    s->ell_ok = s->step_smem_max > 0 &&
+                (s->ell_only || ((B == 32 || B == 64 || (B == 128 && p->x_dtype != DT_F32)) &&
+                                 (p->problem == PROB_MIS ? p->x_dtype != DT_F16 : g->d_w == nullptr)));
     // Default: 16-byte lanes with the ELL stream (the fewest instructions
     // per gathered byte).  MQO_STEP_ELL=1: the ELL stream with the lanes
     // MQO_STEP_KERNEL selects (8-byte unless "wide"); MQO_STEP_KERNEL=wide
@@ -982,6 +988,7 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     const bool ell_forced = ellv && strcmp(ellv, "1") == 0;
     const bool ell_off = ellv && strcmp(ellv, "0") == 0;
     if (!ellv && !force && s->ell_ok && step_wide_possible(B, p->x_dtype)) s->S.step_wide = 1;
+    if (s->ell_only) s->S.step_wide = 1;
     // Dense member graphs: the tensor-core kernel, unless an environment
     // variable above selects one of the others (MQO_STEP_KERNEL=dense: this
     // one where possible).  Its time grows with n per row, theirs with the
@@ -1088,6 +1095,10 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
       }
     }
     if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
+    if (s->ell_only && !s->step_ell) {  // switched off, or its arrays could not be built
+      if (!ell_off && s->step_smem > 0) s->step_smem_max = 0;
+      s->step_smem = 0;
+    }
     // The fused per-graph discrete kernel runs one CTA per member graph, so
     // it is the default only with at least half as many member graphs as
     // SMs; with fewer, the node-parallel passes (several CTAs per item) fill
@@ -1716,13 +1727,13 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
     for (size_t dc : discs) {
       if (st > 0) {
         for (int c16 : {0, 1}) {
-          if (c16 && !s->g->d_col16) continue;
+          if (s->ell_only || (c16 && !s->g->d_col16)) continue;
           plans.push_back({st, 0, 0, dc, 0, 0, c16, 0, 0});
           if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, c16, 0, 0});
         }
         if (s->ell_ok) {
-          if (S.p.x_dtype != DT_F32) plans.push_back({st, 0, 0, dc, 0, 0, 0, 1, 0});
-          if (wide_ok) plans.push_back({st, 0, 1, dc, 0, 0, 0, 1, 0});
+          if (S.p.x_dtype != DT_F32 && !s->ell_only) plans.push_back({st, 0, 0, dc, 0, 0, 0, 1, 0});
+          if (wide_ok || s->ell_only) plans.push_back({st, 0, 1, dc, 0, 0, 0, 1, 0});
         }
       } else {
         for (int v : {1, 2, 4, 8}) {

@@ -18,14 +18,14 @@ cudaError_t launch_smem_ell(const StepArgs& a, bool wide, size_t smem, bool mis,
 // the row-group kernel (mqo_step_rows.cu)
 cudaError_t launch_step_rows(const StepArgs& a, int x_dtype, int v_dtype, int sms, cudaStream_t s);
 
-// the same for float32 x (mqo_step_f32.cu)
+// the same for float32 x, and for B < 32 (mqo_step_f32.cu)
 cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const int4* ell, const int2* ell_pos,
-                                int grid, cudaStream_t s);
+                                int grid, int x_dtype, int v_dtype, cudaStream_t s);
 
 size_t step_smem_bytes(int B, int x_dtype, int problem, int max_ng) {
-  const size_t sx = x_dtype == DT_F32 ? 4 : 2;
+  const size_t sx = x_dtype == DT_F32 || B < 32 ? 4 : 2;  // below 32 trajectories x is staged as float32
   const size_t rowb = (size_t)B * sx;
-  const size_t pitch = rowb == 64 ? 128 : rowb;
+  const size_t pitch = sx == 2 && rowb == 64 ? 128 : rowb;
   const size_t xb = ((size_t)(max_ng + 1) * pitch + 15) & ~(size_t)15;
   const size_t zb = problem == PROB_MIS ? (((size_t)(max_ng + 1) * ((B + 31) / 32) * 4 + 15) & ~(size_t)15) : 0;
   return xb + zb + ((3 * (size_t)B * 8 + 15) & ~(size_t)15) + (size_t)kItemMaxNodes * 16;
@@ -88,7 +88,7 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
   const bool wide = S.step_wide != 0;
   const bool mis = S.p.problem == PROB_MIS;
   const int grid = S.g.num_items;
-  if (ell && xd == DT_F32) return launch_smem_f32_ell(a, smem, mis, ell, ell_pos, grid, stream);
+  if (ell && (xd == DT_F32 || S.B < 32)) return launch_smem_f32_ell(a, smem, mis, ell, ell_pos, grid, xd, vd, stream);
   if (ell) return launch_smem_ell(a, wide, smem, mis, ell, ell_pos, grid, xd, vd, stream);
   if (xd == DT_F32) return launch_tv<float, float>(wide, smem, mis, a, grid, stream);
   if (xd == DT_BF16 && vd == DT_BF16) return launch_tv<__nv_bfloat16, __nv_bfloat16>(wide, smem, mis, a, grid, stream);

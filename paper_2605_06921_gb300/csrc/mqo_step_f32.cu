@@ -1,6 +1,7 @@
 // mqo_step_f32.cu -- the shared-memory step kernel with the sliced-ELL
-// neighbour stream (the layout is described in mqo_step_smem.cuh) for float32
-// x: MIS, and MaxCut without weights.  The step itself (gradient, momentum,
+// neighbour stream (the layout is described in mqo_step_smem.cuh) on x staged as
+// float32: float32 x, and 16-bit x of fewer than 32 trajectories (widening is
+// exact); MIS, and MaxCut without weights.  The step itself (gradient, momentum,
 // projection, rounding, exact evaluation) is the one of mqo_step.cuh.
 //
 // Bound: the shared-memory reads of the neighbours' rows, 128 bytes per clock
@@ -13,7 +14,10 @@
 // Measured (step, 512 graphs of about 750 nodes, degree 112, B = 32, MIS): 248 us
 // against 308 of the CSR form with 8-byte lanes and 272 with 16-byte ones (145 us
 // are the reads' floor; 90 % of the cycles are taken: 71 % by them, 19 % by the
-// offsets' loads); 400 nodes, degree 8: 27 against 37 and 30.
+// offsets' loads); 400 nodes, degree 8: 27 against 37 and 30.  Below 32
+// trajectories it replaces the staged and global-memory kernels: 345 graphs of 300
+// nodes, degree 150, B = 16: 85 us against 387 and 266 (BF16 83 against 232 and 211),
+// B = 4: 47 against 126 and 196; 400 graphs, degree 6, B = 16: 27 against 36 and 45.
 #include "mqo_step.cuh"
 
 namespace mqo {
@@ -21,7 +25,7 @@ namespace mqo {
 constexpr int kF32Threads = 512;  // two CTAs per SM
 
 // LPR = B / 4 lanes per row, 32 / LPR rows per warp in lockstep
-template <int LPR, bool MIS>
+template <typename TX, typename TV, int LPR, bool MIS>
 __global__ void __launch_bounds__(kF32Threads, 2)
     k_step_f(StepArgs a, const int4* __restrict__ ell, const int2* __restrict__ ell_pos) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -40,17 +44,22 @@ __global__ void __launch_bounds__(kF32Threads, 2)
   const int nrows = item.v1 - item.v0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int nwarps = kF32Threads / 32;
-  const float* __restrict__ Xc = static_cast<const float*>((t & 1) ? a.X1 : a.X0);
-  float* __restrict__ Xn = static_cast<float*>((t & 1) ? a.X0 : a.X1);
+  const TX* __restrict__ Xc = static_cast<const TX*>((t & 1) ? a.X1 : a.X0);
+  TX* __restrict__ Xn = static_cast<TX*>((t & 1) ? a.X0 : a.X1);
   uint32_t* __restrict__ Zn = (t & 1) ? a.ZX0 : a.ZX1;
-  float* __restrict__ V = static_cast<float*>(a.V);
+  TV* __restrict__ V = static_cast<TV*>(a.V);
 
   // stage the member graph's block of x and the zero row of the dummy neighbour
   {
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(Xc + (int64_t)off * B);
+    const TX* src = Xc + (int64_t)off * B;
     for (int i = threadIdx.x; i < ng * PER; i += kF32Threads) {
-      const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem + 16 * i);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src + 16 * (int64_t)i) : "memory");
+      if constexpr (sizeof(TX) == 4) {
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem + 16 * i);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src + 4 * (int64_t)i) : "memory");
+      } else {
+        const Pack<TX, 4> q = ld_pack<TX, 4>(src + 4 * (int64_t)i);
+        *reinterpret_cast<float4*>(smem + 16 * i) = make_float4(to_f(q.e[0]), to_f(q.e[1]), to_f(q.e[2]), to_f(q.e[3]));
+      }
     }
     if (threadIdx.x < PER) reinterpret_cast<int4*>(smem + (size_t)ng * PITCH)[threadIdx.x] = make_int4(0, 0, 0, 0);
     for (int i = threadIdx.x; i < 3 * B; i += kF32Threads) s_cnt[i] = 0ull;
@@ -95,7 +104,8 @@ __global__ void __launch_bounds__(kF32Threads, 2)
     const int4 row = s_rows[has ? vb + sub : vb];
     const int v = row.x;
     const int64_t base = (int64_t)v * B + b0;
-    const float4 vv = has ? __ldcs(reinterpret_cast<const float4*>(V + base)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    Pack<TV, 4> vv{};
+    if (has) vv = ld_pack_stream<TV, 4>(V + base);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     float nb[4] = {0.f, 0.f, 0.f, 0.f};  // MIS: maximum of the neighbours' x; MaxCut: their number in the set
     auto add = [&](int o) {
@@ -139,17 +149,18 @@ __global__ void __launch_bounds__(kF32Threads, 2)
     if (c + 2 < nvec) add4(e2);
     first_vectors(vb + nwarps * RPW);
 
-    const float4 xv = *reinterpret_cast<const float4*>(sXl + (size_t)(v - off) * PITCH);
-    const float xi[4] = {xv.x, xv.y, xv.z, xv.w}, vi[4] = {vv.x, vv.y, vv.z, vv.w};
-    float xo[4], vo[4];
+    Pack<TX, 4> xv, xo;
+    Pack<TV, 4> vo;
+    if constexpr (sizeof(TX) == 4) xv = *reinterpret_cast<const Pack<TX, 4>*>(sXl + (size_t)(v - off) * PITCH);
+    else xv = ld_pack<TX, 4>(Xc + base);
     unsigned zbits = 0u;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       bool zn;
       int d0 = 0, d1 = 0, d2 = 0;
       const int pos = MIS ? (int)(nb[e] > 0.5f) : (int)nb[e];
-      step_element<float, float>(a, MIS, thr, lo, xi[e], vi[e], acc[e], pos, row.w, (stepm >> e) & 1u, xo[e], vo[e], zn,
-                                 d0, d1, d2);
+      step_element<TX, TV>(a, MIS, thr, lo, xv.e[e], vv.e[e], acc[e], pos, row.w, (stepm >> e) & 1u, xo.e[e], vo.e[e],
+                           zn, d0, d1, d2);
       if (has) {
         if constexpr (MIS) {
           cp[e] += (uint32_t)d0 | ((uint32_t)d1 << 10) | ((uint32_t)d2 << 20);
@@ -161,13 +172,13 @@ __global__ void __launch_bounds__(kF32Threads, 2)
       zbits |= (unsigned)zn << e;
     }
     if (has) {
-      *reinterpret_cast<float4*>(Xn + base) = make_float4(xo[0], xo[1], xo[2], xo[3]);
-      *reinterpret_cast<float4*>(V + base) = make_float4(vo[0], vo[1], vo[2], vo[3]);
+      st_pack<TX, 4>(Xn + base, xo);
+      st_pack<TV, 4>(V + base, vo);
     }
     unsigned word = zbits << (b0 & 31);
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
-    if (has && (l & 7) == 0) Zn[(int64_t)v * BW + (b0 >> 5)] = word;
+    for (int o = 1; o < (LPR < 8 ? LPR : 8); o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
+    if (has && l % 8 == 0) Zn[(int64_t)v * BW + (b0 >> 5)] = word;
   }
   int c1[4], c2[4];
 #pragma unroll
@@ -180,7 +191,7 @@ __global__ void __launch_bounds__(kF32Threads, 2)
 }
 
 cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const int4* ell, const int2* ell_pos,
-                                int grid, cudaStream_t s) {
+                                int grid, int x_dtype, int v_dtype, cudaStream_t s) {
   if (!mis && a.g.w != nullptr) return cudaErrorInvalidValue;  // the stream carries no weights
   auto run = [&](auto kern) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -188,8 +199,23 @@ cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const 
     kern<<<grid, kF32Threads, smem, s>>>(a, ell, ell_pos);
     return cudaGetLastError();
   };
-  if (a.B == 32) return mis ? run(k_step_f<8, true>) : run(k_step_f<8, false>);
-  if (a.B == 64) return mis ? run(k_step_f<16, true>) : run(k_step_f<16, false>);
+  auto go = [&](auto tx, auto tv) -> cudaError_t {
+    using TX = decltype(tx);
+    using TV = decltype(tv);
+    if (a.B == 4) return mis ? run(k_step_f<TX, TV, 1, true>) : run(k_step_f<TX, TV, 1, false>);
+    if (a.B == 8) return mis ? run(k_step_f<TX, TV, 2, true>) : run(k_step_f<TX, TV, 2, false>);
+    if (a.B == 16) return mis ? run(k_step_f<TX, TV, 4, true>) : run(k_step_f<TX, TV, 4, false>);
+    if constexpr (std::is_same<TX, float>::value) {
+      if (a.B == 32) return mis ? run(k_step_f<TX, TV, 8, true>) : run(k_step_f<TX, TV, 8, false>);
+      if (a.B == 64) return mis ? run(k_step_f<TX, TV, 16, true>) : run(k_step_f<TX, TV, 16, false>);
+    }
+    return cudaErrorInvalidValue;
+  };
+  if (x_dtype == DT_F32) return go(float{}, float{});
+  if (x_dtype == DT_BF16 && v_dtype == DT_BF16) return go(__nv_bfloat16{}, __nv_bfloat16{});
+  if (x_dtype == DT_BF16 && v_dtype == DT_F32) return go(__nv_bfloat16{}, float{});
+  if (x_dtype == DT_F16 && v_dtype == DT_F16) return go(__half{}, __half{});
+  if (x_dtype == DT_F16 && v_dtype == DT_F32) return go(__half{}, float{});
   return cudaErrorInvalidValue;
 }
 

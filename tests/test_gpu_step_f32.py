@@ -1,7 +1,7 @@
-"""The float32 shared-memory step kernel with the sliced-ELL stream against
-the plain global-memory kernel: the same steps, statistics and bits, for rows
-of 0, 1 and many entries, items of 1 to 256 rows, and x out of the box or not
-a number."""
+"""The shared-memory step kernel with the sliced-ELL stream for float32 x, and
+for every type below 32 trajectories, against the plain global-memory kernel:
+the same steps, statistics and bits, for rows of 0, 1 and many entries, items
+of 1 to 256 rows, and x out of the box or not a number."""
 import numpy as np
 import pytest
 
@@ -27,9 +27,10 @@ def packed():
 
 
 @pytest.mark.parametrize("problem,objective", [(0, 0), (1, 0), (1, 2)])
-@pytest.mark.parametrize("B", [32, 64])
+@pytest.mark.parametrize("B,xd,vd", [(b, 0, 0) for b in (4, 8, 16, 32, 64)]
+                         + [(4, 1, 1), (8, 2, 2), (16, 1, 0), (16, 2, 0), (16, 1, 1), (4, 2, 0)])
 @pytest.mark.parametrize("special", [None, float("nan"), float("inf"), -0.0, 1e-30])
-def test_f32_step_equals_generic(mq, monkeypatch, problem, objective, B, special):
+def test_f32_step_equals_generic(mq, monkeypatch, problem, objective, B, xd, vd, special):
     monkeypatch.setenv("MQO_TICK_KERNEL", "ticks")
     G = packed()
     gen = torch.Generator(device="cuda").manual_seed(B)
@@ -42,11 +43,11 @@ def test_f32_step_equals_generic(mq, monkeypatch, problem, objective, B, special
             monkeypatch.setenv("MQO_STEP_KERNEL", force)
         else:
             monkeypatch.delenv("MQO_STEP_KERNEL", raising=False)
-        s = mq.Solver(mq.Graph(G), mq.params(problem=problem, objective=objective, batch=B, gamma=1.7, lambda_=0.3,
-                                             alpha=0.8 if problem == 0 else 0.02, momentum=0.4))
+        s = mq.Solver(mq.Graph(G), mq.params(problem=problem, objective=objective, batch=B, x_dtype=xd, v_dtype=vd,
+                                             gamma=1.7, lambda_=0.3, alpha=0.8 if problem == 0 else 0.02, momentum=0.4))
         info = s.info()
         assert (info["step_kernel"], info["ell"]) == (("global", False) if force else ("smem_wide", True))
-        s.set_x(x0)
+        s.set_x(x0.to([torch.float32, torch.bfloat16, torch.float16][xd]))
         s.step(1 if special is not None else 5)
         out.append([s.get_x(), s.get_v(), *s.step_stats(), s.round()])
     for p, q in zip(*out):
