@@ -307,7 +307,7 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * padded to a common length, four neighbour offsets per 16-byte vector;
  * MIS with bfloat16 or float32 x, or unweighted MaxCut; every type for 4 to
  * 16 trajectories, whose x it stages as float32; about 4 bytes of device
- * memory per entry and lane width), bit 18 = the tensor-core kernel
+ * memory per entry and lane width, 2 for float32 x and below 32 trajectories), bit 18 = the tensor-core kernel
  * of dense member graphs (bit 0 is set too: it keeps x in shared memory),
  * bit 19 = mqo_run and mqo_step take many ticks per launch, one CTA per
  * member graph (small graphs; the other bits describe the plan of single

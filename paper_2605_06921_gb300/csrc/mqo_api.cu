@@ -665,6 +665,7 @@ mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
   ell_shape(s->S.B, s->S.p.x_dtype, wide, &rpw, &pitch);
   for (const auto& es : s->ell_sets)
     if (es.rpw == rpw && es.pitch == pitch) return es;
+  const bool e16 = s->S.p.x_dtype == DT_F32 || s->S.B < 32;  // eight 16-bit entries per vector
   mqo_solver_s::EllSet es;
   es.rpw = rpw;
   es.pitch = pitch;
@@ -681,12 +682,12 @@ mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
       }
       const int32_t nvec = (dmax + 3) / 4;
       for (int32_t p = p0; p < p1; ++p) pos[(size_t)p] = make_int2((int32_t)std::min<int64_t>(total, INT32_MAX), nvec);
-      total += (int64_t)nvec * rpw;
+      total += (int64_t)(e16 ? (nvec + 1) / 2 : nvec) * rpw;
     }
   if (total < INT32_MAX && dalloc(&es.d, (size_t)total, &s->allocs) == MQO_OK &&
       dalloc(&es.pos, (size_t)g->n, &s->allocs) == MQO_OK &&
       cudaMemcpy(es.pos, pos.data(), sizeof(int2) * (size_t)g->n, cudaMemcpyHostToDevice) == cudaSuccess &&
-      launch_ell_fill(g->dev(), rpw, pitch, es.pos, es.d, s->work) == cudaSuccess &&
+      (e16 ? launch_ell_fill16 : launch_ell_fill)(g->dev(), rpw, pitch, es.pos, es.d, s->work) == cudaSuccess &&
       cudaStreamSynchronize(s->work) == cudaSuccess)
     es.ok = true;
   else

@@ -36,6 +36,8 @@ struct DensePlan {
 cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const int2* tiles, int num_tiles,
                               uint4* bits, cudaStream_t s);
 size_t dense_smem_bytes(int max_ng);
+// the stream of x staged as float32 (mqo_step_f32.cu): 16-bit entries
+cudaError_t launch_ell_fill16(const GraphDev& g, int rpw, int pitch, const int2* pos, int4* ell, cudaStream_t s);
 bool step_wide_possible(int B, int x_dtype);
 // the row-group kernel (mqo_step_rows.cu)
 bool step_rows_possible(int B, int x_dtype, int problem, int objective, int max_degree);

@@ -7,17 +7,18 @@
 // Bound: the shared-memory reads of the neighbours' rows, 128 bytes per clock
 // and SM.  The CSR form of k_step_s also takes a shuffle per neighbour and,
 // for MIS, reads rounding words, both through the same path.  Here a lane holds
-// four trajectories (one 16-byte read per neighbour), the neighbours' byte
-// offsets come four at a time from global memory, and the checker's counts
-// come from the gathered values: MIS takes their maximum, MaxCut adds 1.0f for
-// each positive one (exact up to 2^24).
-// Measured (step, 512 graphs of about 750 nodes, degree 112, B = 32, MIS): 248 us
-// against 308 of the CSR form with 8-byte lanes and 272 with 16-byte ones (145 us
-// are the reads' floor; 90 % of the cycles are taken: 71 % by them, 19 % by the
-// offsets' loads); 400 nodes, degree 8: 27 against 37 and 30.  Below 32
-// trajectories it replaces the staged and global-memory kernels: 345 graphs of 300
-// nodes, degree 150, B = 16: 85 us against 387 and 266 (BF16 83 against 232 and 211),
-// B = 4: 47 against 126 and 196; 400 graphs, degree 6, B = 16: 27 against 36 and 45.
+// four trajectories (one 16-byte read per neighbour), the neighbours' offsets come
+// eight at a time from global memory (16 bits each: a vector's load takes four
+// wavefronts of that path although eight lanes read the same 16 bytes), and the
+// checker's counts come from the gathered values: MIS takes their maximum, MaxCut
+// adds 1.0f for each positive one (exact up to 2^24).
+// Measured (step, 512 graphs of about 750 nodes, degree 112, B = 32, MIS): 217 us
+// against 308 of the CSR form with 8-byte lanes and 272 with 16-byte ones, and 248
+// with four 32-bit offsets per vector (145 us are the reads' floor); 400 nodes,
+// degree 8: 27 against 37 and 30.  Below 32 trajectories it replaces the staged
+// and global-memory kernels: 345 graphs of 300 nodes, degree 150, B = 16: 78 us
+// against 386 and 269 (BF16 79 against 233 and 209), B = 4: 39 against 126 and 196;
+// 400 graphs, degree 6, B = 16: 26 against 34 and 44.
 #include "mqo_step.cuh"
 
 namespace mqo {
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(kF32Threads, 2)
   const int32_t ng = a.g.node_off[g + 1] - off;
   const size_t xbytes = (size_t)(ng + 1) * PITCH;
   unsigned long long* s_cnt = reinterpret_cast<unsigned long long*>(smem + xbytes);
-  // the item's rows in processing order: {node, group's first vector, group's nvec, degree}
+  // the item's rows in processing order: {node, group's first vector, its half vectors per row, degree}
   int4* s_rows = reinterpret_cast<int4*>(smem + xbytes + 3 * (size_t)B * 8);
   const int nrows = item.v1 - item.v0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -82,11 +83,12 @@ __global__ void __launch_bounds__(kF32Threads, 2)
   // MIS: all three counts packed in cp (below 2^10 per lane); MaxCut: the last two
   int c0[4] = {0, 0, 0, 0};
   uint32_t cp[4] = {0u, 0u, 0u, 0u};
-  const int dummy = ng * PITCH;
+  // two entries of the dummy neighbour: offsets in units of 16 bytes
+  const int dummy = ng * LPR * 0x00010001;
   const int4 none = make_int4(dummy, dummy, dummy, dummy);
 
-  // a ring of four vectors of a group: 0 and 1 are loaded during the previous
-  // group's tail, each is refilled four vectors ahead once it is summed
+  // a ring of two vectors (eight entries each) of a group: loaded during the
+  // previous group's tail, refilled two vectors ahead once summed
   int4 e0 = none, e1 = none;
   auto first_vectors = [&](int i) {
     e0 = e1 = none;
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(kF32Threads, 2)
       const int4 r = s_rows[i];
       const int4* p = ell + r.y + sub;
       if (r.z > 0) e0 = __ldcs(p);
-      if (r.z > 1) e1 = __ldcs(p + RPW);
+      if (r.z > 2) e1 = __ldcs(p + RPW);
     }
   };
   first_vectors(warp * RPW);
@@ -122,31 +124,23 @@ __global__ void __launch_bounds__(kF32Threads, 2)
         add_f32x2(nb[2], nb[3], f.z > 0.f ? 1.f : 0.f, f.w > 0.f ? 1.f : 0.f);
       }
     };
-    auto add4 = [&](const int4& q) {
-      add(q.x);
-      add(q.y);
-      add(q.z);
-      add(q.w);
+    auto add2 = [&](int w) {
+      add((w & 0xffff) << 4);
+      add((int)((uint32_t)w >> 16) << 4);
     };
-    const int nvec = grp.z;
+    const int nhalf = grp.z;  // halves (four entries) of vectors
     const int4* ep = ell + grp.y + sub;
-    int4 e2 = none, e3 = none;
-    if (nvec > 2) e2 = __ldcs(ep + 2 * RPW);
-    if (nvec > 3) e3 = __ldcs(ep + 3 * RPW);
     int c = 0;
-    for (; c + 4 <= nvec; c += 4) {
-      add4(e0);
-      if (c + 4 < nvec) e0 = __ldcs(ep + (c + 4) * RPW);
-      add4(e1);
-      if (c + 5 < nvec) e1 = __ldcs(ep + (c + 5) * RPW);
-      add4(e2);
-      if (c + 6 < nvec) e2 = __ldcs(ep + (c + 6) * RPW);
-      add4(e3);
-      if (c + 7 < nvec) e3 = __ldcs(ep + (c + 7) * RPW);
+    for (; c + 4 <= nhalf; c += 4) {
+      const int4 q0 = e0, q1 = e1;
+      if (c + 4 < nhalf) e0 = __ldcs(ep + (c / 2 + 2) * RPW);
+      add2(q0.x), add2(q0.y), add2(q0.z), add2(q0.w);
+      if (c + 6 < nhalf) e1 = __ldcs(ep + (c / 2 + 3) * RPW);
+      add2(q1.x), add2(q1.y), add2(q1.z), add2(q1.w);
     }
-    if (c < nvec) add4(e0);
-    if (c + 1 < nvec) add4(e1);
-    if (c + 2 < nvec) add4(e2);
+    if (c < nhalf) add2(e0.x), add2(e0.y);
+    if (c + 1 < nhalf) add2(e0.z), add2(e0.w);
+    if (c + 2 < nhalf) add2(e1.x), add2(e1.y);
     first_vectors(vb + nwarps * RPW);
 
     Pack<TX, 4> xv, xo;
@@ -188,6 +182,44 @@ __global__ void __launch_bounds__(kF32Threads, 2)
     c2[e] = (int)(cp[e] >> 20);
   }
   flush_step_counters<4>(a, s_cnt, g, it, b0, LPR, c0, c1, c2, stepm);
+}
+
+// The stream: as k_ell_fill (mqo_step_ell.cu) with eight 16-bit entries per
+// vector, offsets in units of 16 bytes (an x block is at most 110 KB); pos[..].y
+// counts half vectors, and the second half of a group's last vector may be unused.
+__global__ void k_ell_fill16(GraphDev g, int rpw, int lpr, const int2* __restrict__ pos, int4* __restrict__ ell) {
+  const Item item = g.items[blockIdx.x];
+  const int nrows = item.v1 - item.v0;
+  const int32_t off = g.node_off[item.g];
+  const int dummy = (g.node_off[item.g + 1] - off) * lpr;
+  const int ngrp = (nrows + rpw - 1) / rpw;
+  for (int i = threadIdx.x; i < ngrp * rpw; i += blockDim.x) {
+    const int q = i / rpw, r = i - q * rpw;
+    const int2 ep = pos[item.v0 + q * rpw];
+    int rs = 0, re = 0;
+    if (i < nrows) {
+      const int v = g.order[item.v0 + i];
+      rs = g.row_ptr[v];
+      re = g.row_ptr[v + 1];
+    }
+    for (int c = 0; c < (ep.y + 1) / 2; ++c) {
+      int e[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int j = rs + 8 * c + 2 * k;
+        const int lo = j < re ? (g.col[j] - off) * lpr : dummy;
+        const int hi = j + 1 < re ? (g.col[j + 1] - off) * lpr : dummy;
+        e[k] = lo | (hi << 16);
+      }
+      ell[(int64_t)ep.x + (int64_t)c * rpw + r] = make_int4(e[0], e[1], e[2], e[3]);
+    }
+  }
+}
+
+cudaError_t launch_ell_fill16(const GraphDev& g, int rpw, int pitch, const int2* pos, int4* ell, cudaStream_t s) {
+  if (g.num_items <= 0) return cudaSuccess;
+  k_ell_fill16<<<g.num_items, 256, 0, s>>>(g, rpw, pitch / 16, pos, ell);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const int4* ell, const int2* ell_pos,
