@@ -626,8 +626,8 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
     read and written once, rounding words) per launch over its average
     launch time; the shared-memory kernel adds its gather bound."""
     # index bytes per CSR entry: 16-bit member-local ids, 32-bit ids, or the
-    # sliced-ELL stream's 32-bit row offsets (its padding not counted)
-    idx = 4 if plan.get("ell") else (2 if plan.get("col16") else 4)
+    # sliced-ELL stream's row offsets (its padding not counted; float32 x: 16 bits)
+    idx = (2 if x_dtype == "f32" else 4) if plan.get("ell") else (2 if plan.get("col16") else 4)
     alg = algorithmic_bytes_per_step(G, B, sx, sv, idx)
     if plan.get("dense"):  # bit matrices (rows and columns padded to 128) in place of the column indices
         rows = -(-member_sizes(G) // 128) * 128
