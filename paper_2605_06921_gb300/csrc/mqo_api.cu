@@ -1094,6 +1094,18 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         s->step_smem = 0;
         s->S.step_staged = 2;
       }
+      // float32 x: the staged kernel copies every neighbour row through shared
+      // memory, where 512-byte rows leave a slice few of them, and long steps wait
+      // for the copies' issue; the global-memory kernel reads the rows from L2.  Measured
+      // (staged against global, us): B = 128: 10^4 nodes, degree 10 (51 MB of neighbour
+      // rows) 31 and 31, degree 40 123 and 58, 10^6 nodes, degree 12 2636 and 1889;
+      // B = 64: 3 10^4 nodes, degree 20 (154 MB) 61 and 74, 10^5, degree 30 (769 MB) 271
+      // and 198; B = 32: 10^5, degree 30 (384 MB) 133 and 117; x of 128 MB and more
+      // 688 and 854.
+      const double gathered = (double)g->nnz * B * 4;
+      const bool direct = (B == 128 && gathered >= 50e6) ||
+                          ((B == 32 || B == 64) && gathered >= 300e6 && g->n * B * 4 <= kL2Bytes / 2);
+      if (none_forced && p->x_dtype == DT_F32 && s->S.step_staged == 1 && covered && direct) s->S.step_staged = 0;
     }
     if (s->step_smem > 0 && !s->dense) use_ell(s, ell_forced || (!ell_off && !force));
     if (s->ell_only && !s->step_ell) {  // switched off, or its arrays could not be built

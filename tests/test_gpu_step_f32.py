@@ -55,3 +55,22 @@ def test_f32_step_equals_generic(mq, monkeypatch, problem, objective, B, xd, vd,
             assert bool(((p == q) | (torch.isnan(p) & torch.isnan(q))).all())
         else:
             assert torch.equal(p, q)
+
+
+def test_f32_step_default_outside_shared_memory(mq, monkeypatch):
+    """long steps of wide float32 rows read them from L2, short ones and narrow rows are staged; the same steps"""
+    for name in ("MQO_STEP_KERNEL", "MQO_STEP_ELL", "MQO_COL16"):
+        monkeypatch.delenv(name, raising=False)
+    G = mq.Graph(mi.erdos_renyi(10000, 0.002, 1))
+    out = []
+    for B, force, kern in ((128, None, "global"), (128, "staged", "staged"), (64, None, "staged")):
+        if force:
+            monkeypatch.setenv("MQO_STEP_KERNEL", force)
+        else:
+            monkeypatch.delenv("MQO_STEP_KERNEL", raising=False)
+        s = mq.Solver(G, mq.params(batch=B, seed=3))
+        assert s.info()["step_kernel"] == kern
+        s.init()
+        s.step(3)
+        out.append(s.get_x())
+    assert torch.equal(out[0], out[1])
