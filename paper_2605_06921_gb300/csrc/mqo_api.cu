@@ -44,7 +44,7 @@ constexpr int kSmallTicks = 4096;               // ticks per launch of that kern
 constexpr int kDenseMaxDegree = 1023;  // tensor-core step: neighbour counts take 10 bits
 constexpr size_t kDenseSmemLimit = 225 * 1024;  // and 32 trajectories of a member graph's x fit in shared memory
 constexpr int64_t kL2Bytes = (int64_t)129 << 20;
-constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3 bytes per CSR entry at most)
+constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3.1 bytes per CSR entry at most)
 constexpr int kDefaultSliceKB = 32;  // staged step kernel: gathered x rows per slice (KB)
 
 }  // namespace
@@ -173,6 +173,7 @@ template <typename T>
 mqo_status dalloc(T** p, size_t count, std::vector<void*>* track) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch
   if (e != cudaSuccess) return fail(MQO_ENOMEM, "cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
   *p = static_cast<T*>(q);
   if (track) track->push_back(q);
@@ -311,7 +312,8 @@ mqo_status validate(int64_t n, int64_t nnz, const int64_t* rp, const int32_t* co
 // Bit matrices of the member graphs (mqo_step_dense.cuh) where the step of
 // dense member graphs may use them: no weights, degrees that fit the
 // companion counts, an x block of 32 trajectories that fits in shared memory,
-// and at least kDenseFill of the matrices' cells set.
+// and at least kDenseFill of the matrices' cells set.  They only make calls
+// faster: where there is no memory for them the graph stays without.
 mqo_status build_dense_bits(mqo_graph g, const std::vector<int32_t>& dmax, cudaStream_t stream) {
   for (int32_t k = 0; k < g->G; ++k) {
     g->max_ng = std::max(g->max_ng, g->h_off[(size_t)k + 1] - g->h_off[(size_t)k]);
@@ -334,8 +336,11 @@ mqo_status build_dense_bits(mqo_graph g, const std::vector<int32_t>& dmax, cudaS
   if (st == MQO_OK) st = dalloc(&g->d_bits_off, (size_t)g->G, nullptr);
   if (st == MQO_OK) st = dalloc(&d_tiles, tiles.size(), nullptr);
   if (st != MQO_OK) {
-    cudaFree(d_tiles);
-    return st;
+    cudaFree(g->d_bits);
+    cudaFree(g->d_bits_off);
+    g->d_bits = nullptr;
+    g->d_bits_off = nullptr;
+    return MQO_OK;
   }
   cudaError_t e = cudaMemcpy(g->d_bits_off, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice);
