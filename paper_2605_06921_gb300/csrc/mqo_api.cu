@@ -37,12 +37,8 @@ mqo_status fail(mqo_status st, const char* fmt, ...) {
 
 constexpr int kChunkNodes = kItemMaxNodes;  // nodes per item
 constexpr int kSplit = 512;       // row length above which the f_B kernels chunk a row
-constexpr size_t kStepSmemLimit = 110 * 1024;  // shared-memory step kernel if the graph block fits
-constexpr size_t kDiscSmemLimit = 160 * 1024;  // fused discrete kernel if the graph's bit words fit
-constexpr size_t kSmallSmemLimit = 200 * 1024;  // multi-tick kernel: a member graph and its trajectories fit
 constexpr int kSmallTicks = 4096;               // ticks per launch of that kernel
 constexpr int kDenseMaxDegree = 1023;  // tensor-core step: neighbour counts take 10 bits
-constexpr size_t kDenseSmemLimit = 225 * 1024;  // and 32 trajectories of a member graph's x fit in shared memory
 constexpr int64_t kL2Bytes = (int64_t)129 << 20;
 constexpr double kDenseFill = 0.04;    // and this share of the bit matrices' cells is set (3.1 bytes per CSR entry at most)
 constexpr int kDefaultSliceKB = 32;  // staged step kernel: gathered x rows per slice (KB)
@@ -626,7 +622,7 @@ mqo_solver_s::SliceSet slice_set(mqo_solver s, int cap_kb) {
   const size_t smem = staged_layout(s->S.B, (int)dtype_size(s->S.p.x_dtype), (int)dtype_size(s->S.p.v_dtype), ss.cols,
                                     ss.rows, true)
                           .total;
-  if (smem > 200 * 1024 || !build_slices(s->g, ss.rows, ss.cols, h) || h.empty()) {
+  if (smem > kStagedSmemLimit || !build_slices(s->g, ss.rows, ss.cols, h) || h.empty()) {
     ss.count = -1;
   } else if (dalloc(&ss.d, h.size(), &s->allocs) != MQO_OK ||
              cudaMemcpy(ss.d, h.data(), h.size() * sizeof(Slice), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -1131,6 +1127,7 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     // Member graphs with bit matrices: the form that follows the trajectories in
     // a round (MQO_DISC_KERNEL=bits where possible; the others exclude it).
     s->disc_bits_max = g->d_bits != nullptr && B >= 32 ? disc_bits_smem_bytes(p->problem, max_ng) : 0;
+    if (s->disc_bits_max > kDiscBitsSmemLimit) s->disc_bits_max = 0;
     if (s->disc_bits_max > 0 && (!dforce || strcmp(dforce, "bits") == 0)) {
       s->disc_bits = true;
       s->disc_smem = s->disc_bits_max;

@@ -503,7 +503,7 @@ cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_
   // a CTA per word, 7.3 with one per graph)
   int parts = S.Bw;
   while (parts > 1 && S.g.num_graphs * parts > sms) parts /= 2;
-  cudaError_t e = cudaFuncSetAttribute(k_disc_bits, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_disc_bits, kDiscBitsSmemLimit);
   if (e != cudaSuccess) return e;
   k_disc_bits<<<S.g.num_graphs * parts, kDbThreads, smem, stream>>>(S, bits, bits_off);
   return cudaGetLastError();

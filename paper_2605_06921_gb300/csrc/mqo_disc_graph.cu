@@ -414,7 +414,8 @@ size_t disc_graph_smem_bytes(int B, int max_ng) {
 }
 
 cudaError_t launch_disc_graph(const SolverDev& S, size_t smem, cudaStream_t stream) {
-  cudaFuncSetAttribute(k_disc_graph, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_disc_graph, kDiscSmemLimit);
+  if (e != cudaSuccess) return e;
   k_disc_graph<<<S.g.num_graphs, kDgThreads, smem, stream>>>(S);
   return cudaGetLastError();
 }

@@ -10,6 +10,21 @@ namespace mqo {
 
 constexpr int kPairThreads = 256;  // pair kernels: (node, trajectory) per thread
 
+// The most dynamic shared memory a plan may ask of each kind of kernel, and
+// what every launch of such a kernel allows it (allow_smem): the same value
+// whatever the solver, so that host threads whose solvers need different
+// amounts do not lower each other's limit between the call and the launch.
+constexpr size_t kStepSmemLimit = 110 * 1024;     // shared-memory step kernels: the member graph's block fits
+constexpr size_t kDiscSmemLimit = 160 * 1024;     // fused discrete kernel: the member graph's bit words fit
+constexpr size_t kDiscBitsSmemLimit = 120 * 1024; // its form on bit matrices
+constexpr size_t kSmallSmemLimit = 200 * 1024;    // multi-tick kernel: a member graph and its trajectories fit
+constexpr size_t kStagedSmemLimit = 200 * 1024;   // staged-gather step kernel: a slice fits
+constexpr size_t kDenseSmemLimit = 224 * 1024;    // tensor-core step: 32 trajectories of a member graph's x fit
+template <typename K>
+inline cudaError_t allow_smem(K kern, size_t limit) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
+
 enum CtrlMode : int { CTRL_MACHINE = 0, CTRL_LS_BEGIN = 1, CTRL_LS = 2, CTRL_RESET = 3 };
 
 struct DensePlan;

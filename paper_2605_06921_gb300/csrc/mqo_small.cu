@@ -291,7 +291,7 @@ __global__ void k_tick_add(int64_t* tick, int64_t n) { *tick += n; }
 
 cudaError_t launch_small(const SolverDev& S, int count, Counters* plain, int threads, size_t smem, cudaStream_t s) {
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kSmallSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<S.g.num_graphs, threads, smem, s>>>(S, count, plain);
     k_tick_add<<<1, 1, 0, s>>>(S.tick, (int64_t)count);

@@ -860,7 +860,7 @@ size_t dense_smem_bytes(int max_ng) {
 template <typename TX, typename TV>
 static cudaError_t launch_t(const StepArgs& a, const DenseArgs& d, int grid, size_t smem, cudaStream_t s) {
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kDenseSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<grid, kDenseThreads + 32, smem, s>>>(a, d);
     return cudaGetLastError();

@@ -226,7 +226,7 @@ cudaError_t launch_smem_f32_ell(const StepArgs& a, size_t smem, bool mis, const 
                                 int grid, int x_dtype, int v_dtype, cudaStream_t s) {
   if (!mis && a.g.w != nullptr) return cudaErrorInvalidValue;  // the stream carries no weights
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kStepSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<grid, kF32Threads, smem, s>>>(a, ell, ell_pos);
     return cudaGetLastError();

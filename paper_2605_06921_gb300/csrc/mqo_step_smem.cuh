@@ -433,7 +433,8 @@ static cudaError_t launch_s(size_t smem, const StepArgs& a, const int4* ell, con
                             cudaStream_t s) {
   if (a.B != VEC * LPR) return cudaErrorInvalidValue;
   auto kern = k_step_s<TX, TV, VEC, LPR, MIS, DUP, ELL>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(kern, kStepSmemLimit);
+  if (e != cudaSuccess) return e;
   kern<<<grid, kStepNT<VEC, ELL>, smem, s>>>(a, ell, ell_pos);
   return cudaGetLastError();
 }

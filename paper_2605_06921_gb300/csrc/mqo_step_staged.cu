@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kStagedThreads, VEC >= 8 ? 2 : 4) k_step_q(Ste
 template <typename TX, typename TV, int VEC>
 static cudaError_t launch_q_vec(const StepArgs& a, size_t smem, cudaStream_t s) {
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kStagedSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<a.num_slices, kStagedThreads, smem, s>>>(a);
     return cudaGetLastError();
