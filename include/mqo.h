@@ -14,8 +14,13 @@
  * Conventions for every entry point:
  *  - Status: every call returns an mqo_status; no C++ exception crosses
  *    the ABI.  mqo_last_error() returns a thread-local message for the last
- *    failure on the calling thread.  After MQO_ECUDA the solver is poisoned
- *    and later calls on it return MQO_ESTATE.
+ *    failure on the calling thread.  After MQO_ECUDA or MQO_ETIMEOUT the
+ *    solver is poisoned and later calls on it return MQO_ESTATE.
+ *    MQO_ETIMEOUT: a wait inside a step kernel ran out, that step and later
+ *    ones of the solver stored nothing for the member graphs concerned, and
+ *    outputs read since hold no valid iterate.  The first call on the solver
+ *    that finds the kernel's mark reports it, whichever call it is; those
+ *    that synchronise look again after their wait.
  *  - Streams: `cuda_stream` is a cudaStream_t passed as void* (NULL = the
  *    legacy default stream).  Work is enqueued asynchronously unless the
  *    call says it synchronises.
@@ -55,7 +60,7 @@ typedef enum {
   MQO_EGRAPH = -2,  /* CSR failed validation (see mqo_last_error) */
   MQO_ENOMEM = -3,  /* device or host allocation failed */
   MQO_ECUDA = -4,   /* a CUDA call failed; the solver is poisoned */
-  MQO_ETIMEOUT = -5,/* a bounded wait inside a step kernel ran out (reported by mqo_best and mqo_traj_state) */
+  MQO_ETIMEOUT = -5,/* a bounded wait inside a step kernel ran out; the solver is poisoned */
   MQO_ESTATE = -6   /* solver poisoned by an earlier failure */
 } mqo_status;
 

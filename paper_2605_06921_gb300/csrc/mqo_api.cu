@@ -125,6 +125,7 @@ struct mqo_solver_s {
   Counters* d_eval = nullptr;
   int32_t* h_pending = nullptr;  // pinned
   int32_t* d_pending = nullptr;
+  int32_t* h_late = nullptr;  // pinned; set by a step kernel whose wait ran out
   // saved state around a standalone local search
   void* d_save = nullptr;
   std::vector<void*> allocs;
@@ -604,10 +605,25 @@ mqo_status poison(mqo_solver s, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return poison(s, e_, #call); \
   } while (0)
 
+// A wait of the step kernel ran out: what it left is no step.
+mqo_status look_late(mqo_solver s) {
+  if (!s->h_late || *static_cast<volatile int32_t*>(s->h_late) == 0) return MQO_OK;
+  s->poisoned = true;
+  return fail(MQO_ETIMEOUT, "a wait of the step kernel ran out");
+}
+
+// after the work the caller waits for
+#define CHECK_LATE(s)                                  \
+  do {                                                 \
+    const mqo_status late_ = look_late(s);             \
+    if (late_ != MQO_OK) return late_;                 \
+  } while (0)
+
 #define CHECK_SOLVER(s)                                                             \
   do {                                                                              \
     if (!(s)) return fail(MQO_EINVAL, "null solver");                               \
     if ((s)->poisoned) return fail(MQO_ESTATE, "solver poisoned by an earlier error"); \
+    CHECK_LATE(s);                                                                  \
   } while (0)
 
 // The staged kernel's slices for `cap_kb` KB of gathered x rows, built and
@@ -1154,7 +1170,14 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
   if ((st = dalloc(&S.gflag, (size_t)3 * g->G, &s->allocs)) != MQO_OK) return bail(st);
   if ((st = dalloc(&S.any, 4, &s->allocs)) != MQO_OK) return bail(st);
   if ((st = dalloc(&s->d_pending, 1, &s->allocs)) != MQO_OK) return bail(st);
-  if (cudaMallocHost(&s->h_pending, sizeof(int32_t)) != cudaSuccess) return bail(fail(MQO_ENOMEM, "pinned alloc"));
+  if ((st = dalloc(&s->dense_plan.late, 1, &s->allocs)) != MQO_OK) return bail(st);
+  if (cudaMallocHost(&s->h_pending, 2 * sizeof(int32_t)) != cudaSuccess) return bail(fail(MQO_ENOMEM, "pinned alloc"));
+  s->h_late = s->h_pending + 1;
+  *s->h_late = 0;
+  s->dense_plan.host_late = s->h_late;
+  // MQO_DENSE_POLLS: the looks of a wait inside the tensor-core step (0: every wait runs out)
+  const char* polls = getenv("MQO_DENSE_POLLS");
+  s->dense_plan.polls = polls ? (uint32_t)std::min<unsigned long>(strtoul(polls, nullptr, 10), kDensePolls) : kDensePolls;
   {
     // node-parallel kernels take several CTAs per item when there are few
     // items, so that about four CTAs' worth of nodes reach every SM
@@ -1167,6 +1190,7 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     cudaMemsetAsync(S.tick, 0, sizeof(int64_t), s->work);
     cudaMemsetAsync(S.gflag, 0, sizeof(int32_t) * 3 * g->G, s->work);
     cudaMemsetAsync(S.any, 0, sizeof(int32_t) * 4, s->work);
+    cudaMemsetAsync(s->dense_plan.late, 0, sizeof(int32_t), s->work);
     cudaMemsetAsync(x1, 0, s->x_bytes, s->work);
     cudaEventRecord(s->ev_out, s->work);
     cudaStreamWaitEvent(s->user, s->ev_out, 0);
@@ -1291,6 +1315,7 @@ mqo_status mqo_run_timed(mqo_solver s, int64_t nticks, double* phase_ms, int64_t
   }
   for (auto& e : ev) cudaEventDestroy(e);
   if (err != cudaSuccess) return poison(s, err, "mqo_run_timed");
+  CHECK_LATE(s);
   s->host_tick += nticks;
   if (phase_ms)
     for (int p = 0; p < kPhases; ++p) phase_ms[p] = tot[p];
@@ -1405,6 +1430,7 @@ mqo_status mqo_local_search(mqo_solver s, int32_t max_rounds) {
     CKS(launch_any_pending(S, s->d_pending, s->work));
     CKS(cudaMemcpyAsync(s->h_pending, s->d_pending, sizeof(int32_t), cudaMemcpyDeviceToHost, s->work));
     CKS(cudaStreamSynchronize(s->work));
+    CHECK_LATE(s);
     if (*s->h_pending == 0) break;
   }
   if (ticks & 1) {  // keep the parity of the x buffers
@@ -1421,19 +1447,14 @@ mqo_status mqo_best(mqo_solver s, int64_t* values, uint32_t* z_bits) {
   CHECK_SOLVER(s);
   const SolverDev& S = s->S;
   const size_t T = (size_t)S.g.num_graphs * S.B;
-  *s->h_pending = 0;
   {
     Scope sc(s);
-    if (s->dense) CKS(cudaMemcpyAsync(s->h_pending, S.any + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, s->work));
     if (z_bits) CKS(cudaMemcpyAsync(z_bits, S.Zbest, s->words * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s->work));
     if (values) CKS(cudaMemcpyAsync(values, S.bestv, T * sizeof(int64_t), cudaMemcpyDeviceToHost, s->work));
   }
   CKS(cudaStreamSynchronize(s->work));
   CKS(cudaStreamSynchronize(s->user));
-  if (*s->h_pending) {
-    s->poisoned = true;
-    return fail(MQO_ETIMEOUT, "a wait of the step kernel ran out");
-  }
+  CHECK_LATE(s);
   return MQO_OK;
 }
 
@@ -1478,6 +1499,7 @@ mqo_status mqo_pool_state(mqo_solver s, int32_t* counts, int64_t* values, int64_
   }
   CKS(cudaStreamSynchronize(s->work));
   CKS(cudaStreamSynchronize(s->user));
+  CHECK_LATE(s);
   for (int g = 0; g < G; ++g) {
     if (counts) counts[g] = ps[(size_t)g].count;
     if (merges) merges[g] = ps[(size_t)g].merges;
@@ -1496,14 +1518,7 @@ mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out) {
   CKS(cudaStreamSynchronize(s->work));
   CKS(cudaMemcpy(h.data(), s->S.st, T * sizeof(TrajState), cudaMemcpyDeviceToHost));
   CKS(cudaMemcpy(c.data(), s->S.cnt, T * R * sizeof(Counters), cudaMemcpyDeviceToHost));
-  if (s->dense) {
-    int32_t late = 0;
-    CKS(cudaMemcpy(&late, s->S.any + 3, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    if (late) {
-      s->poisoned = true;
-      return fail(MQO_ETIMEOUT, "a wait of the step kernel ran out");
-    }
-  }
+  CHECK_LATE(s);
   const bool mis = s->p.problem == MQO_MIS;
   for (size_t i = 0; i < T; ++i) {
     // the counters of the last tick are folded into the state by the next
@@ -1866,6 +1881,10 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
   if (err != cudaSuccess) {
     apply(keep);
     return poison(s, err, "mqo_autotune");
+  }
+  if (look_late(s) != MQO_OK) {
+    apply(keep);
+    return MQO_ETIMEOUT;
   }
   apply(chosen);
   // the captured tick graphs hold the old launch configuration

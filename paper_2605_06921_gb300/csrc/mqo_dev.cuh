@@ -160,7 +160,7 @@ struct SolverDev {
   Counters* cnt;    // [G*B*R]
   int64_t* tick;    // current tick number
   int32_t* gflag;   // [3*G] tick stamps: any apply / any discrete / any step
-  int32_t* any;     // [4] per-tick "any trajectory" stamps (apply, disc, step); [3]: a wait of the step kernel ran out
+  int32_t* any;     // [4] per-tick "any trajectory" stamps (apply, disc, step)
   int64_t* bestv;   // [G*B] best value of each trajectory (compact copy for readout)
   // pool mode (p.pool_k = K > 0)
   int32_t K, Kw;    // pool size, pool bit words per node

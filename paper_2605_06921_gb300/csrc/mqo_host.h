@@ -40,13 +40,20 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
 cudaError_t launch_ell_fill(const GraphDev& g, int rpw, int pitch, const int2* pos, int4* ell, cudaStream_t s);
 // dense member graphs on the tensor cores (mqo_step_dense.cuh): their bit
 // matrices, the CTAs per (member graph, 32 trajectories), the dynamic shared
-// memory of a CTA and the bits of the largest degree (degree < 2^sum_bits)
+// memory of a CTA and the bits of the largest degree (degree < 2^sum_bits);
+// the looks of a wait inside the kernel before it gives up, and the words that
+// are set then: the step's later CTAs and launches see the device's and do
+// nothing, the host reads its own
+constexpr uint32_t kDensePolls = 1u << 27;
 struct DensePlan {
   const uint4* bits;
   const int64_t* bits_off;  // per member graph: first uint4
   int32_t parts;
   int32_t sum_bits;
   size_t smem;
+  uint32_t polls;
+  int32_t* late;
+  int32_t* host_late;
 };
 cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const int2* tiles, int num_tiles,
                               uint4* bits, cudaStream_t s);

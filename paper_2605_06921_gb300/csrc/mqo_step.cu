@@ -68,7 +68,7 @@ cudaError_t launch_step(const SolverDev& S, Counters* cnt, const int32_t* act, c
   a.slice_rows = S.slice_rows;
   a.slice_cols = S.slice_cols;
   const int xd = S.p.x_dtype, vd = S.p.v_dtype;
-  if (dense) return launch_step_dense(a, *dense, S.any + 3, xd, vd, stream);
+  if (dense) return launch_step_dense(a, *dense, xd, vd, stream);
   if (smem == 0 && S.step_staged == 2) return launch_step_rows(a, xd, vd, sms, stream);
   if (smem == 0 && S.step_staged) {
     // staged-gather kernel: one CTA per slice

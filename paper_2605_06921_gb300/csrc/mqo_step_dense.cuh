@@ -55,11 +55,11 @@ struct DenseArgs {
   float t0, t1;               // |x| >= t0: exact up to the largest degree; >= t1: up to s1
   float s1x2;                 // 2 * s1
   float degree;               // mean degree of all member graphs
-  int32_t* err;               // set if a wait ran out
+  volatile int32_t* late;       // set if a wait ran out (device memory)
+  volatile int32_t* host_late;  // the same, in pinned host memory
+  uint32_t polls;               // looks of a wait
 };
 
-// `err` is set if a wait of the kernel ran out
-cudaError_t launch_step_dense(const StepArgs& a, const DensePlan& p, int32_t* err, int x_dtype, int v_dtype,
-                              cudaStream_t s);
+cudaError_t launch_step_dense(const StepArgs& a, const DensePlan& p, int x_dtype, int v_dtype, cudaStream_t s);
 
 }  // namespace mqo
