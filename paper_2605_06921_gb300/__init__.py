@@ -450,6 +450,7 @@ def _autograd():
         @staticmethod
         def backward(ctx, gout):
             _, ax = ctx.saved_tensors
+            ax = ax.contiguous()  # saved-tensor hooks may give another layout back
             B = ax.shape[1]
             G = torch.empty_like(ax)
             g = gout.to(torch.float32).contiguous()
