@@ -422,16 +422,11 @@ def pga_adam_step(x, m, u, grad, lr, b1, b2, eps, t, lo, hi):
 def _autograd():
     import torch
 
-    class FbObjective(torch.autograd.Function):
+    class FbFunction(torch.autograd.Function):
         """f_B(X) per column (Eq. 7).  Where a gradient may be asked for, the
         forward keeps A X and the backward forms the gradient from it (one
         gather for both); X is saved too, so that a change of it in place
         between the two is still an error."""
-
-        @classmethod
-        def apply(cls, X, graph, lambda_):
-            # the grad mode is off inside forward
-            return super().apply(X, graph, lambda_, torch.is_grad_enabled())
 
         @staticmethod
         def forward(ctx, X, graph, lambda_, grad_enabled):
@@ -457,6 +452,15 @@ def _autograd():
             _check(lib().mqo_fb_grad_ax(ctx.graph.handle, _dptr(ax), _dptr(g), _dptr(G), B, float(ctx.lambda_),
                                         _stream()))
             return G, None, None, None
+
+    class FbObjective(FbFunction):
+        __doc__ = FbFunction.__doc__
+
+        # no super() here: torch.compile cannot trace it in a Function's apply
+        @staticmethod
+        def apply(X, graph, lambda_):
+            # the grad mode is off inside forward
+            return FbFunction.apply(X, graph, lambda_, torch.is_grad_enabled())
 
     class PGAMomentum(torch.optim.Optimizer):
         """Projected momentum ascent on p.grad: v <- mu v + g, p <- Pi(p + lr v)."""
