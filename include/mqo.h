@@ -16,11 +16,10 @@
  *    the ABI.  mqo_last_error() returns a thread-local message for the last
  *    failure on the calling thread.  After MQO_ECUDA or MQO_ETIMEOUT the
  *    solver is poisoned and later calls on it return MQO_ESTATE.
- *    MQO_ETIMEOUT: a wait inside a step kernel ran out, that step and later
- *    ones of the solver stored nothing for the member graphs concerned, and
- *    outputs read since hold no valid iterate.  The first call on the solver
- *    that finds the kernel's mark reports it, whichever call it is; those
- *    that synchronise look again after their wait.
+ *    MQO_ETIMEOUT: a wait inside a step kernel ran out, and what that step
+ *    and later ones left is void, also in outputs enqueued since.  The first
+ *    call on the solver that finds the kernel's mark reports it, whichever
+ *    call it is; those that synchronise look again after their wait.
  *  - Streams: `cuda_stream` is a cudaStream_t passed as void* (NULL = the
  *    legacy default stream).  Work is enqueued asynchronously unless the
  *    call says it synchronises.

@@ -605,7 +605,7 @@ mqo_status poison(mqo_solver s, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return poison(s, e_, #call); \
   } while (0)
 
-// A wait of the step kernel ran out: what it left is no step.
+// A wait of the step kernel ran out: the x and V it left are no step's.
 mqo_status look_late(mqo_solver s) {
   if (!s->h_late || *static_cast<volatile int32_t*>(s->h_late) == 0) return MQO_OK;
   s->poisoned = true;
@@ -1170,11 +1170,10 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
   if ((st = dalloc(&S.gflag, (size_t)3 * g->G, &s->allocs)) != MQO_OK) return bail(st);
   if ((st = dalloc(&S.any, 4, &s->allocs)) != MQO_OK) return bail(st);
   if ((st = dalloc(&s->d_pending, 1, &s->allocs)) != MQO_OK) return bail(st);
-  if ((st = dalloc(&s->dense_plan.late, 1, &s->allocs)) != MQO_OK) return bail(st);
   if (cudaMallocHost(&s->h_pending, 2 * sizeof(int32_t)) != cudaSuccess) return bail(fail(MQO_ENOMEM, "pinned alloc"));
   s->h_late = s->h_pending + 1;
   *s->h_late = 0;
-  s->dense_plan.host_late = s->h_late;
+  s->dense_plan.late = s->h_late;
   // MQO_DENSE_POLLS: the looks of a wait inside the tensor-core step (0: every wait runs out)
   const char* polls = getenv("MQO_DENSE_POLLS");
   s->dense_plan.polls = polls ? (uint32_t)std::min<unsigned long>(strtoul(polls, nullptr, 10), kDensePolls) : kDensePolls;
@@ -1190,7 +1189,6 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     cudaMemsetAsync(S.tick, 0, sizeof(int64_t), s->work);
     cudaMemsetAsync(S.gflag, 0, sizeof(int32_t) * 3 * g->G, s->work);
     cudaMemsetAsync(S.any, 0, sizeof(int32_t) * 4, s->work);
-    cudaMemsetAsync(s->dense_plan.late, 0, sizeof(int32_t), s->work);
     cudaMemsetAsync(x1, 0, s->x_bytes, s->work);
     cudaEventRecord(s->ev_out, s->work);
     cudaStreamWaitEvent(s->user, s->ev_out, 0);

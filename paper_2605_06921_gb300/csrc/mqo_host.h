@@ -41,10 +41,9 @@ cudaError_t launch_ell_fill(const GraphDev& g, int rpw, int pitch, const int2* p
 // dense member graphs on the tensor cores (mqo_step_dense.cuh): their bit
 // matrices, the CTAs per (member graph, 32 trajectories), the dynamic shared
 // memory of a CTA and the bits of the largest degree (degree < 2^sum_bits);
-// the looks of a wait inside the kernel before it gives up, and the words that
-// are set then: the step's later CTAs and launches see the device's and do
-// nothing, the host reads its own
-constexpr uint32_t kDensePolls = 1u << 27;
+// the looks of a wait inside the kernel before it gives up, and the word in
+// pinned host memory that it sets then
+constexpr uint32_t kDensePolls = 1u << 26;
 struct DensePlan {
   const uint4* bits;
   const int64_t* bits_off;  // per member graph: first uint4
@@ -53,7 +52,6 @@ struct DensePlan {
   size_t smem;
   uint32_t polls;
   int32_t* late;
-  int32_t* host_late;
 };
 cudaError_t launch_dense_bits(const GraphDev& g, const int64_t* bits_off, const int2* tiles, int num_tiles,
                               uint4* bits, cudaStream_t s);

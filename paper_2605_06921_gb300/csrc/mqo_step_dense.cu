@@ -62,11 +62,12 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-// false if the phase has not ended after `polls` looks (a wait is a few
-// microseconds, kDensePolls looks about two seconds of running; time in which
-// the context is not scheduled does not count)
+// false if the phase has not ended after `polls` looks (looked at every 256;
+// a wait is a few microseconds, kDensePolls looks about a second of running, in
+// which time without the context on the GPU does not count)
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t polls) {
-  for (uint32_t i = 0; i < polls; ++i) {
+#pragma unroll 1
+  for (uint32_t i = 0;; ++i) {
     uint32_t ok;
     asm volatile("{\n\t.reg .pred p;\n\t"
                  "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -75,8 +76,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
                  : "r"(bar), "r"(parity)
                  : "memory");
     if (ok) return true;
+    if ((i & 255u) == 255u) {
+      if (i >= polls) return false;
+      asm volatile("" ::: "memory");  // keeps the test out of the look's path
+    }
   }
-  return false;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -218,9 +222,7 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
   using T2 = typename X::T2;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t s_mbar[2][4];  // per warpgroup: A buffers 0 / 1 written, MMAs done with 0 / 1
-  __shared__ __align__(8) uint64_t s_drain;       // all MMAs done, after a wait has run out
   __shared__ uint32_t s_tmem;
-  __shared__ int s_late;                          // an earlier CTA's wait ran out
   __shared__ uint32_t s_cnt[3][32];
   __shared__ uint16_t s_list[kDoubtful];  // doubtful pairs: node << 5 | trajectory bit
   __shared__ int s_listed;
@@ -255,9 +257,7 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 32 * kIssuer) {
-    s_late = *d.late;
     for (int i = 0; i < 8; ++i) mbar_init(smem_addr(&s_mbar[i >> 2][i & 3]), (i & 2) ? 1 : 4);
-    mbar_init(smem_addr(&s_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 96) s_cnt[tid >> 5][tid & 31] = 0u;
@@ -387,26 +387,20 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
   const uint32_t stepw = __ballot_sync(0xffffffffu, (myact & ACT_STEP) != 0);
   uint32_t n0 = 0u, n1 = 0u, n2 = 0u;  // counts of trajectory traj_of_bit(lane)
   uint32_t use[2] = {0u, 0u};          // chunks that went through each A buffer
-  // a wait ran out, here or in an earlier CTA: no more waits, nothing is stored
-  bool dead = s_late != 0;
-  bool issued = false;
-  const bool lead = warp == kIssuer && elect_one();  // issues the MMAs
+  bool dead = d.polls == 0u;           // a wait ran out: no more waits; this block's results are void
   if (warp == kIssuer) {
     // Issues the MMAs of both warpgroups, chunk by chunk as they are written,
     // in a fixed order (few instructions: the warp shares its scheduler).  An
     // MMA instruction waits for the tensor pipe (32 cycles each at N = 64), so
     // a warp that also expands would hold its warpgroup up.
-    if (!heavy && lead) {
+    if (!heavy && elect_one()) {
       const uint32_t full0 = smem_addr(&s_mbar[0][0]);
       const uint64_t bd0 = bdesc0;
       uint32_t ph = 0u;  // bit 2 w + buf: phase of the warpgroup's written barrier
       auto issue = [&](int w, int buf, int c, int nk) {
         const uint32_t full = full0 + 32u * w + 8u * buf;
-        if (dead || !mbar_wait(full, (ph >> (2 * w + buf)) & 1u, d.polls)) {
-          dead = true;  // the warpgroups' waits for these MMAs run out too
-          return;
-        }
-        issued = true;
+        if (!dead && !mbar_wait(full, (ph >> (2 * w + buf)) & 1u, d.polls)) dead = true;
+        if (dead) return;  // the warpgroups' waits for these MMAs run out too
         ph ^= 1u << (2 * w + buf);
         tc_fence_after();
         const uint32_t dd = tmem0 + 128u * w, ab = dd + 64u + 32u * buf;
@@ -417,9 +411,9 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
         if (nk > 3) mma_ts(dd, ab + 24u, bd + 384u, idesc, 1u);
         mma_commit(full + 16u);
       };
-      for (int tile0 = 2 * part; tile0 < tiles && !dead; tile0 += 2 * d.parts) {
+      for (int tile0 = 2 * part; tile0 < tiles; tile0 += 2 * d.parts) {
         const bool both = tile0 + 1 < tiles;
-        for (int c = 0; c < n64 && !dead; c += 2) {
+        for (int c = 0; c < n64; c += 2) {
           const int nk = nk16 - 4 * c;
           issue(0, 0, c, nk);
           if (both) issue(1, 0, c, nk);
@@ -429,6 +423,9 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
           }
         }
       }
+      // none is in flight when the block ends, also where a wait has run out
+      for (int i = 0; i < 4; ++i)
+        if (!mbar_wait(full0 + 16u + 32u * (i >> 1) + 8u * (i & 1), ((ph >> i) & 1u) ^ 1u, kDensePolls)) dead = true;
     }
     __syncwarp();
   }
@@ -597,7 +594,7 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
       }
     }
   };
-  for (int tile = 2 * part + wg; warp != kIssuer && tile < tiles && !dead; tile += 2 * d.parts) {
+  for (int tile = 2 * part + wg; warp != kIssuer && tile < tiles; tile += 2 * d.parts) {
     const int vl = tile * 128 + wtid;
     const bool has = vl < ng;
     const uint4* bp = bits0 + (int64_t)tile * tiles * 128;
@@ -640,8 +637,6 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
     const int deg = MIS ? 0 : a.g.row_ptr[off + (has ? vl : 0) + 1] - a.g.row_ptr[off + (has ? vl : 0)];
     if (use[0] > 0 && !dead && !mbar_wait(bar + 16u, (use[0] - 1) & 1u, d.polls)) dead = true;
     if (use[1] > 0 && !dead && !mbar_wait(bar + 24u, (use[1] - 1) & 1u, d.polls)) dead = true;
-    dead = __any_sync(0xffffffffu, dead) != 0;
-    if (dead) break;
     tc_fence_after();
 
     // Which pairs are doubtful?  Few go on the list; a warp with many sums its
@@ -832,18 +827,7 @@ __global__ void __launch_bounds__(kDenseThreads + 32, 2) k_step_t(StepArgs a, De
     if (n1) atomicAdd(&s_cnt[1][b], n1);
     if (n2) atomicAdd(&s_cnt[2][b], n2);
   }
-  if (dead) {
-    // the MMAs in flight still read this block's memory
-    if (lead && issued) {
-      mma_commit(smem_addr(&s_drain));
-      mbar_wait(smem_addr(&s_drain), 0u, kDensePolls);
-    }
-    if (tid == 0) {
-      *d.late = 1;
-      *d.host_late = 1;
-      __threadfence_system();
-    }
-  }
+  if (dead) *d.late = 1;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -904,7 +888,6 @@ cudaError_t launch_step_dense(const StepArgs& a, const DensePlan& p, int x_dtype
   d.t1 = ldexpf(1.0f, -t - 4);
   d.s1x2 = ldexpf(2.0f, s0 - 4);
   d.late = p.late;
-  d.host_late = p.host_late;
   d.polls = p.polls;
   d.degree = (float)((double)a.g.nnz / (double)a.g.n);
   const int grid = a.g.num_graphs * d.groups * d.parts;

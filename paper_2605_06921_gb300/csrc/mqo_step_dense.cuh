@@ -55,8 +55,7 @@ struct DenseArgs {
   float t0, t1;               // |x| >= t0: exact up to the largest degree; >= t1: up to s1
   float s1x2;                 // 2 * s1
   float degree;               // mean degree of all member graphs
-  volatile int32_t* late;       // set if a wait ran out (device memory)
-  volatile int32_t* host_late;  // the same, in pinned host memory
+  volatile int32_t* late;       // set if a wait ran out (pinned host memory)
   uint32_t polls;               // looks of a wait
 };
 

@@ -1,7 +1,7 @@
 """A wait inside the tensor-core step kernel that runs out: every call on the
 solver reports it once the kernel has marked it, the calls that synchronise
-at once, and the context stays usable.  MQO_DENSE_POLLS=0 makes every wait
-run out at its first look."""
+at once, and the context stays usable.  MQO_DENSE_POLLS=0: every wait has run
+out before its first look."""
 import pytest
 
 import mqo_inputs as mi
