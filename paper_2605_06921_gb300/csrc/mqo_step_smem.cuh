@@ -41,11 +41,16 @@ namespace mqo {
 //    The next group's vectors are prefetched into L2 while the current
 //    group is summed.
 
-// add_bf16_row plus a running maximum of the row's bfloat16 bit patterns read
-// as signed 16-bit integers, one 32-bit word (two trajectories) per mx[]
-// entry.  For bfloat16 values in [0, 1] that order is the order of the
-// values, and -0 (0x8000) reads as the most negative: after a row, half k of
-// mx[w] > 0x3F00 (= 0.5) iff some neighbour of trajectory 2w + k has x > 0.5.
+// add_bf16_row plus a running maximum of the row's bfloat16 values from 0 up,
+// one 32-bit word (two trajectories) per mx[] entry: after a row, half k of
+// mx[w], read as an integer, is > 0x3F00 (= 0.5) iff some neighbour of
+// trajectory 2w + k has x > 0.5.  A NaN is left out (the other operand is the
+// maximum), as it is not in the set.
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
 template <int VEC>
 __device__ __forceinline__ void add_bf16_row_max(float* acc, uint32_t* mx, const unsigned char* p);
 template <>
@@ -53,8 +58,8 @@ __device__ __forceinline__ void add_bf16_row_max<4>(float* acc, uint32_t* mx, co
   const uint2 r = *reinterpret_cast<const uint2*>(p);
   add_bf16x2_word(acc[0], acc[1], r.x);
   add_bf16x2_word(acc[2], acc[3], r.y);
-  mx[0] = __vmaxs2(mx[0], r.x);
-  mx[1] = __vmaxs2(mx[1], r.y);
+  mx[0] = max_bf16x2(mx[0], r.x);
+  mx[1] = max_bf16x2(mx[1], r.y);
 }
 template <>
 __device__ __forceinline__ void add_bf16_row_max<8>(float* acc, uint32_t* mx, const unsigned char* p) {
@@ -63,14 +68,14 @@ __device__ __forceinline__ void add_bf16_row_max<8>(float* acc, uint32_t* mx, co
   add_bf16x2_word(acc[2], acc[3], r.y);
   add_bf16x2_word(acc[4], acc[5], r.z);
   add_bf16x2_word(acc[6], acc[7], r.w);
-  mx[0] = __vmaxs2(mx[0], r.x);
-  mx[1] = __vmaxs2(mx[1], r.y);
-  mx[2] = __vmaxs2(mx[2], r.z);
-  mx[3] = __vmaxs2(mx[3], r.w);
+  mx[0] = max_bf16x2(mx[0], r.x);
+  mx[1] = max_bf16x2(mx[1], r.y);
+  mx[2] = max_bf16x2(mx[2], r.z);
+  mx[3] = max_bf16x2(mx[3], r.w);
 }
 
 // MIS with bfloat16 x and 4 or 8 trajectories per lane: the checker's
-// neighbour test comes from a running signed max of the gathered bfloat16
+// neighbour test comes from a running max of the gathered bfloat16
 // words (add_bf16_row_max) instead of the neighbours' rounding words
 template <typename TX, int VEC, bool MIS>
 constexpr bool kMaxCheck = MIS && std::is_same<TX, __nv_bfloat16>::value && (VEC == 4 || VEC == 8);

@@ -57,9 +57,17 @@ __device__ __forceinline__ void add_x16x2_word<__half>(float& a, float& b, uint3
       : "+f"(a), "+f"(b)
       : "r"(w));
 }
-// the 16-bit pattern of 0.5: for values in [0, 1] the patterns read as
-// signed 16-bit integers order like the values (-0 reads as negative), so
-// "some neighbour has x > 0.5" is "the running max of the patterns > it"
+// the running max of a row's values from 0 up, two to a word, and the 16-bit
+// pattern of 0.5: "some neighbour has x > 0.5" is "the max, read as an
+// integer, is above it".  A NaN is left out (the other operand is the
+// maximum), as it is not in the set.
+template <typename TX>
+__device__ __forceinline__ uint32_t max_x16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  if constexpr (std::is_same<TX, __half>::value) asm("max.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  else asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
 template <typename TX>
 constexpr int16_t kHalfPattern = std::is_same<TX, __half>::value ? (int16_t)0x3800 : (int16_t)0x3F00;
 
@@ -156,7 +164,7 @@ __global__ void __launch_bounds__(kStagedThreads, VEC >= 8 ? 2 : 4) k_step_q(Ste
   //    sums are never -0.0), so the sums equal the CSR-order sums and the
   //    loop has no per-row branches.  MIS with 16-bit x: one mixed-precision
   //    add per element, and the checker's "some neighbour in the set" from a
-  //    running signed max of the gathered 16-bit words.
+  //    running max of the gathered 16-bit words.
   constexpr bool kMax16 = MIS && sizeof(TX) == 2 && (VEC == 2 || VEC == 4 || VEC == 8);
   constexpr int NW = VEC / 2 > 0 ? VEC / 2 : 1;  // 32-bit words of a lane's elements
   const unsigned char* zp = s_zero + b0 * (int)sizeof(TX);
@@ -196,7 +204,7 @@ __global__ void __launch_bounds__(kStagedThreads, VEC >= 8 ? 2 : 4) k_step_q(Ste
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
           add_x16x2_word<TX>(acc[2 * w], acc[2 * w + 1], wd[w]);
-          mx[w] = __vmaxs2(mx[w], wd[w]);
+          mx[w] = max_x16x2<TX>(mx[w], wd[w]);
         }
       } else {
         float f[VEC];
