@@ -316,7 +316,9 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * bit 19 = mqo_run and mqo_step take many ticks per launch, one CTA per
  * member graph (small graphs; the other bits describe the plan of single
  * ticks, which mqo_run_timed takes), bit 20 = the row-group kernel (16-bit x,
- * neighbour rows read from L2, bits 0 and 3 clear); *smem_bytes = the
+ * neighbour rows read from L2, bits 0 and 3 clear), bit 21 = the fused
+ * discrete passes run on the bit matrices of dense member graphs (bit 1 is set
+ * too); *smem_bytes = the
  * shared-memory step kernel's dynamic shared memory per CTA; *items = work
  * items (node ranges of at most 256 nodes); *replicas = counter replicas per
  * trajectory.

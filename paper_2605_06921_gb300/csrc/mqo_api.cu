@@ -1474,7 +1474,7 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                    ((staged ? slice_kb(s) : 0) << 8) |
                    ((s->step_smem > 0 && s->S.step_c16 && !s->dense) ? (1 << 16) : 0) |
                    ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0) |
-                   (s->small ? (1 << 19) : 0) | (rows ? (1 << 20) : 0);
+                   (s->small ? (1 << 19) : 0) | (rows ? (1 << 20) : 0) | (s->disc_bits ? (1 << 21) : 0);
   if (smem_bytes) *smem_bytes = (int64_t)(s->dense ? s->dense->smem : s->step_smem);
   if (items) *items = s->S.g.num_items;
   if (replicas) *replicas = s->S.R;
@@ -1900,7 +1900,8 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
                 (chosen.small ? (1 << 19) : 0) | (chosen.disc_smem > 0 ? 2 : 0) | (chosen.wide ? 4 : 0) |
                 (stg ? 8 : 0) | (chosen.vec << 4) | ((stg ? chosen.slice_kb : 0) << 8) |
                 ((chosen.step_smem > 0 && chosen.c16) ? (1 << 16) : 0) |
-                ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0) | (rows ? (1 << 20) : 0);
+                ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0) | (rows ? (1 << 20) : 0) |
+                (chosen.dbits ? (1 << 21) : 0);
   }
   if (best_ms_per_tick) *best_ms_per_tick = best / ticks;
   return MQO_OK;
