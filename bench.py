@@ -10,10 +10,11 @@ evaluation, acceptance, mutation resets, repair and local search).
 Metric: edge-updates/s = CSR entries of the member graph for every
 trajectory tick that ran a gradient step, per second of the timed ticks
 (trajectories in a repair or local-search round that tick are not counted).
-The default line carries sub-records: the steady state, batched against
+The default run also measures the steady state, batched against
 single-instance quality, the other configurations (MaxCut on a 3-regular
 graph, MIS at 10^7 nodes, the f_B autograd workload) and the paper-shaped
-ER workloads.
+ER workloads: the printed line has their value and time, the file
+bench_detail.json beside this one the complete record.
 
 Arms:
   default            the CUDA library (one process per GPU, weak scaling)
@@ -834,10 +835,55 @@ def gpu_arm(args):
         if objective_f64:
             line["objective_f64"] = objective_f64
         line.update(sub)
-        print(json.dumps(line))
+        emit(line)
     if dist is not None:
         dist.destroy_process_group()
     return 0
+
+
+LINE_LIMIT = 2800  # characters of the printed line
+
+
+def short_line(line):
+    """The record as the one printed line: everything but the sub-records and
+    the longer parts of the roofline and the baseline, and value and time of
+    every sub-record; below LINE_LIMIT characters, so that a reader that keeps
+    the end of the output has all of it."""
+    def short(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    out = {k: v for k, v in line.items() if not isinstance(v, (dict, list)) or k in ("config", "e2e", "clocks")}
+    if "e2e" in out:
+        out["e2e"] = {k: v for k, v in out["e2e"].items() if k != "note"}
+    for k in ("roofline", "cpu_baseline", "objective_f64", "kernel_ms_per_step"):
+        if k in line:
+            out[k] = {a: short(b) for a, b in line[k].items() if not isinstance(b, (dict, list, bool)) and
+                      not (isinstance(b, str) and len(b) > 40)}
+    steady = line.get("steady_state")
+    if steady:
+        out["steady_state"] = {k: short(steady[k]) for k in ("value_median", "ms_per_step_median") if k in steady}
+    out["configs"] = {k: {a: short(v[a]) for a in ("value", "ms_per_step") if a in v}
+                      for k, v in line.get("configs", {}).items()}
+    if not out["configs"]:
+        del out["configs"]
+    for k in ("configs", "steady_state", "objective_f64", "kernel_ms_per_step", "cpu_baseline", "roofline"):
+        if len(json.dumps(out)) < LINE_LIMIT:
+            break
+        out.pop(k, None)
+    return out
+
+
+def emit(line, path=None):
+    """Prints the short line and keeps the complete record in a file beside
+    this one (bench_detail.json)."""
+    path = os.path.join(ROOT, "bench_detail.json") if path is None else path
+    try:
+        with open(path, "w", encoding="utf-8") as f:
+            json.dump(line, f, indent=1)
+        progress(f"complete record: {path}")
+    except OSError as e:
+        progress(f"complete record not written: {e}")
+    print(json.dumps(short_line(line)), flush=True)
 
 
 def paper_quality(mq, G, wl, pkw, xd, vd, ticks):
@@ -1346,7 +1392,7 @@ def autograd_arm(args):
     line = autograd_measure(mq, args.steps, args.warmup, local=local, rank=rank, dist=dist,
                             cpu=rank == 0 and world == 1 and not args.no_cpu)
     if rank == 0:
-        print(json.dumps(line))
+        emit(line)
     if dist is not None:
         dist.destroy_process_group()
     return 0
