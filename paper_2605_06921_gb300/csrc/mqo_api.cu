@@ -1097,13 +1097,23 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         // Member graphs that fit in shared memory: that kernel runs one CTA per item
         // and leaves the GPU idle below about a third as many items as SMs (n = 300,
         // degree 20, B = 128, MIS: 8 items 34 us against 15 of the staged kernel, 32
-        // items 35 against 23, 100 items 35 against 41).  MaxCut's longer tail moves
-        // its line against the row groups to as many items as SMs, or to a mean degree
-        // of 8 (B = 128: 100 items, degree 20: 53 against 34; 300 items, degree 4: 49
-        // against 38, degree 20: 74 against 76).
+        // items 35 against 23, 100 items 35 against 41).  MaxCut's longer tail moves its
+        // line against the row groups.  They share all rows out over the GPU, so their
+        // time grows with items and degree, the other's with the degree alone.  Row
+        // groups against shared memory, us of a plain step (BF16, n = 400): 72 items,
+        // B = 32, degree 48: 29.6 and 30.0, degree 96: 42 and 38.5; B = 64, degree 96:
+        // 45 and 61; 100 items, B = 64, degree 96: 65 and 61; B = 128, degree 96: 92 and
+        // 108; 128 items, B = 32, degree 16: 23.6 and 23.8, degree 96: 48 and 38.5;
+        // B = 128, degree 32: 59 and 62, degree 64: 94 and 86.  At a mean degree of 8 they
+        // win with many items too (1000 items of 250 nodes, B = 128: 0.83 of the time;
+        // 300 items, B = 32: 1.02).
         const int items = (int)g->h_items.size();
         const bool few = 3 * items < g->sms && (s->staged_ok || rows);
-        const bool cut = p->problem == PROB_MAXCUT && rows && (items < g->sms || g->nnz <= 8 * g->n);
+        const double degree = (double)g->nnz / (double)g->n, load = (double)items / g->sms;
+        const double most = load < 0.5    ? (B == 32 ? 48.0 : 1e9)
+                            : load < 0.75 ? (B == 32 ? 32.0 : B == 64 ? 48.0 : 1e9)
+                                          : B / 4.0;
+        const bool cut = p->problem == PROB_MAXCUT && rows && ((items < g->sms && degree <= most) || degree <= 8.0);
         if (few || cut) s->step_smem = 0;
         else rows = false;
       }
