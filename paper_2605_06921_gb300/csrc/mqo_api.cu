@@ -1097,9 +1097,15 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         // Member graphs that fit in shared memory: that kernel runs one CTA per item
         // and leaves the GPU idle below about a third as many items as SMs (n = 300,
         // degree 20, B = 128, MIS: 8 items 34 us against 15 of the staged kernel, 32
-        // items 35 against 23, 100 items 35 against 41).  MaxCut's longer tail moves its
-        // line against the row groups.  They share all rows out over the GPU, so their
-        // time grows with items and degree, the other's with the degree alone.  Row
+        // items 35 against 23, 100 items 35 against 41), but not where an item has
+        // little to gather (us of a tick with a pool, BF16, MIS: 33 items of 60 nodes,
+        // degree 10, B = 32: 21.5 of the staged kernel against 18.2; 48 items of 30,
+        // degree 4, B = 128: 23.2 against 20.2; 16 items of 60, degree 10, B = 32: 19.3
+        // against 17.1, MaxCut 17.8 and 18.2), nor with float32 x and many long rows (48
+        // items of 250, degree 30, B = 64: 44 against 30; of 60, B = 128: 33.5 against
+        // 26.6).  MaxCut's longer tail moves its line against the row groups.  They share
+        // all rows out over the GPU, so their time grows with items and degree, the
+        // other's with the degree alone.  Row
         // groups against shared memory, us of a plain step (BF16, n = 400): 72 items,
         // B = 32, degree 48: 29.6 and 30.0, degree 96: 42 and 38.5; B = 64, degree 96:
         // 45 and 61; 100 items, B = 64, degree 96: 65 and 61; B = 128, degree 96: 92 and
@@ -1108,12 +1114,18 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         // win with many items too (1000 items of 250 nodes, B = 128: 0.83 of the time;
         // 300 items, B = 32: 1.02).
         const int items = (int)g->h_items.size();
-        const bool few = 3 * items < g->sms && (s->staged_ok || rows);
         const double degree = (double)g->nnz / (double)g->n, load = (double)items / g->sms;
+        const bool f32 = p->x_dtype == DT_F32;
+        const bool mis = p->problem == PROB_MIS;
+        const double least = items <= 32 ? (!mis || B == 128 ? 0.0 : B == 64 ? 20e3 : 28e3)
+                                         : (B == 32 ? (mis ? 50e3 : 30e3) : B == 64 ? 28e3 : f32 ? 0.0 : 31e3);
+        const double gathered = (double)g->nnz * B / items;
+        const bool long_rows = f32 && (B < 128 ? items * degree > 900.0 : items * degree > 1300.0 && gathered < 300e3);
+        const bool few = 3 * items < g->sms && (s->staged_ok || rows) && gathered >= least && !long_rows;
         const double most = load < 0.5    ? (B == 32 ? 48.0 : 1e9)
                             : load < 0.75 ? (B == 32 ? 32.0 : B == 64 ? 48.0 : 1e9)
                                           : B / 4.0;
-        const bool cut = p->problem == PROB_MAXCUT && rows && ((items < g->sms && degree <= most) || degree <= 8.0);
+        const bool cut = !mis && rows && ((items < g->sms && degree <= most) || degree <= 8.0);
         if (few || cut) s->step_smem = 0;
         else rows = false;
       }
