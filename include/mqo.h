@@ -313,9 +313,10 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * 16 trajectories, whose x it stages as float32; about 4 bytes of device
  * memory per entry and lane width, 2 for float32 x and below 32 trajectories), bit 18 = the tensor-core kernel
  * of dense member graphs (bit 0 is set too: it keeps x in shared memory),
- * bit 19 = mqo_run and mqo_step take many ticks per launch, one CTA per
+ * bit 19 = mqo_run takes many ticks per launch, one CTA per
  * member graph (small graphs; the other bits describe the plan of single
- * ticks, which mqo_run_timed takes), bit 20 = the row-group kernel (16-bit x,
+ * ticks, which mqo_run_timed takes; mqo_step takes many steps per launch where
+ * they fit, bit 19 set or not), bit 20 = the row-group kernel (16-bit x,
  * neighbour rows read from L2, bits 0 and 3 clear), bit 21 = the fused
  * discrete passes run on the bit matrices of dense member graphs (bit 1 is set
  * too); *smem_bytes = the

@@ -162,6 +162,7 @@ struct mqo_solver_s {
   size_t small_smem = 0;  // > 0: possible, with this much dynamic shared memory
   int small_threads = 0;
   bool small = false;     // the current plan uses it
+  bool small_step = false;  // plain steps use it, whatever the plan of ticks
 };
 
 namespace {
@@ -713,6 +714,43 @@ mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
   return es;
 }
 
+// Is a tick of the machine in the multi-tick kernel no slower than one of the
+// tick's kernels?  Ticks with discrete rounds cost it more than steps do (a
+// CTA walks all lists of its member graph), so where descents are short, so that
+// rounds follow one another, and for MIS, whose capped descents are repaired,
+// both times are estimated: us of a tick, the multi-tick kernel per wave of CTAs
+// from the largest member graph's nodes, pairs and work, the tick's kernels
+// from all pairs and work.  The coefficients are fitted to 1952 machine runs (14
+// sizes and degrees, 1 to 300 graphs, B = 1 to 128, both problems, descents of 50
+// steps and of 2 and 6; the plan taken is 0.5 % behind the better one on
+// average).  Multi-tick against the tick's kernels, us: n = 200, degree 10, B = 1:
+// 2.0 and 13; MIS, n = 100, degree 10, one graph: B = 16 7.4 and 13, B = 32 15.8 and
+// 13.2 to 15.1, B = 64 33 and 14.7; n = 100, degree 4, B = 64, t_gs = 1, cap 6: 44 and 33.
+bool tick_small_faster(mqo_solver s, const mqo_params& p, int pairs, int64_t work, int waves) {
+  const mqo_graph g = s->g;
+  const bool mis = p.problem == PROB_MIS, bits = g->d_bits != nullptr && p.batch >= 32;
+  const bool rounds = (mis && p.repair && p.descent_cap < 20) ||
+                      (p.local_search && ((int64_t)p.t_gs + 1) * p.descent_cap < 300);
+  if (!mis && !rounds) return true;
+  struct Cost {
+    double base, pair, work, node;                        // multi-tick kernel
+    double kernels, all_narrow, all_wide, all_work, b, n, one;  // tick's kernels (narrow: B < 32; one: largest graph's pairs)
+  };
+  static const Cost kDescent[2] = {{1.5, 1.9e-3, 0.086e-3, 0, 14.5, 13.8e-6, 7.4e-6, 1.1e-6, 0.092, 0, 0},
+                                   {0, 4.5e-3, 0.032e-3, 0, 14.7, 0, 12.8e-6, 0, 0.013, 0, 0.05e-3}};
+  static const Cost kMis[2] = {{3.5, 6.3e-3, 0, 5.4e-3, 21.7, 59e-6, 15.8e-6, 0.1e-6, 0.04, 0, 0.5e-3},
+                               {3.9, 3.9e-3, 0.025e-3, 8.1e-3, 27.5, 0, 33e-6, 0, 0.03, 0, 0}};
+  static const Cost kCut[2] = {{3.0, 5.6e-3, 0.23e-3, 0, 21.2, 51e-6, 21e-6, 2.3e-6, 0.029, 0, 0.84e-3},
+                               {8.7, 6.9e-3, 0.047e-3, 17e-3, 24.9, 0, 42e-6, 0, 0.027, 0.038, 0}};
+  const Cost& c = (!rounds ? kDescent : mis ? kMis : kCut)[bits];
+  const double n = g->max_ng, all = (double)g->n * p.batch, all_work = (double)g->nnz * p.batch;
+  const bool narrow = p.batch < 32;
+  const double small = waves * (c.base + c.pair * pairs + c.work * (double)work + c.node * n);
+  const double ticks = c.kernels + (narrow ? c.all_narrow : c.all_wide) * all + (narrow ? c.all_work * all_work : 0.0) +
+                       c.b * p.batch + c.n * n + c.one * pairs;
+  return small <= ticks;
+}
+
 // selects the CSR (on = false) or the sliced-ELL stream for the current lane
 // width; the CSR one when the ELL arrays are not available
 void use_ell(mqo_solver s, bool on) {
@@ -1065,16 +1103,17 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         s->small_threads = std::min(1024, std::max(128, (pairs + 127) / 128 * 128));
         const char* tk = getenv("MQO_TICK_KERNEL");
         const bool other = force || ellv || c16 || getenv("MQO_DISC_KERNEL") || getenv("MQO_SERIAL_TICK");
-        // Its tick takes about 0.8 us, 0.8 ns per (node, trajectory) pair and
+        // A plain step takes about 0.8 us, 0.8 ns per (node, trajectory) pair and
         // 0.06 ns per (entry, trajectory) pair of the largest member graph, and
-        // there is one CTA per SM; a tick of the kernels takes 11 us and up
-        // (n = 200, B = 1: 1.0 against 11.7; n = 400, degree 24, B = 8: 8.3 against
-        // 12.8; n = 200, degree 24, B = 32: 12.9 against 19.5, 300 graphs 26
-        // against 28; n = 400, degree 24, B = 32: 25 against 21).
+        // there is one CTA per SM; a step of the kernels takes 11 us and up (n = 200,
+        // B = 1: 1.0 against 11.7; n = 400, degree 24, B = 8: 8.3 against 12.8;
+        // n = 200, degree 24, B = 32: 12.9 against 19.5, 300 graphs 26 against 28;
+        // n = 400, degree 24, B = 32: 25 against 21).
         const double us = 0.8 + 0.8e-3 * pairs + 0.06e-3 * (double)work;
         const int waves = (g->G + g->sms - 1) / g->sms;
         const bool faster = us <= 11.0 && us * waves <= 22.0;
-        s->small = tk ? strcmp(tk, "small") == 0 : !other && faster;
+        s->small_step = tk ? strcmp(tk, "small") == 0 : !other && faster;
+        s->small = s->small_step && (tk || tick_small_faster(s, *p, pairs, work, waves));
       }
     }
     // 16-bit x, MIS or MaxCut on f_B: the row-group kernel, unless an environment
@@ -1356,7 +1395,7 @@ mqo_status mqo_step(mqo_solver s, int32_t nsteps) {
   if (nsteps < 0) return fail(MQO_EINVAL, "nsteps < 0");
   Scope sc(s);
   const SolverDev& S = s->S;
-  if (s->small) {
+  if (s->small || s->small_step) {
     for (int32_t left = nsteps; left > 0; left -= kSmallTicks)
       CKS(launch_small(S, std::min(left, kSmallTicks), s->d_cnt_plain, s->small_threads, s->small_smem, s->work));
     s->host_tick += nsteps;
