@@ -1048,13 +1048,28 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     // Dense member graphs: the tensor-core kernel, unless an environment
     // variable above selects one of the others (MQO_STEP_KERNEL=dense: this
     // one where possible).  Its time grows with n per row, theirs with the
-    // degree.  Measured (step of 8 to 256 graphs, B = 32 and 128, BF16): against
-    // the shared-memory kernel it wins from a mean degree of about 32 + n / 20
-    // (n = 256, degree 48: 23 us against 26; n = 800, degree 96: 29 against 34;
-    // degree 48: 45 against 41), against the staged and global ones from
-    // 16 + n / 25 (n = 800, B = 128, degree 48: 47 against 132), except where the
-    // row tiles do not fill the GPU (8 graphs of 1200 nodes, B = 32, degree 64,
-    // MaxCut: 38 against 31).
+    // degree, and it works in row tiles of 128 times groups of 32 trajectories,
+    // which have to fill the GPU.  Measured (BF16, us of a step among 8 or 64 graphs
+    // after some ticks, other kernel in brackets):
+    //  * MIS against the shared-memory kernel from a mean degree of 32 + n / 20
+    //    (n = 400, 64 graphs, B = 32, degree 48: 19.5 (20.6); n = 800, degree 64: 28.5
+    //    (28.9), degree 96: 28.8 (33.4)), with fewer tiles than SMs from 38 + n / 18
+    //    (ticks, 16 graphs: n = 600, degree 64 1.13 of the other's time, 100: 0.9);
+    //  * MIS where x does not fit there, against the staged and row-group kernels,
+    //    from 16 + n / 25 (64 graphs, B = 128: n = 600, degree 48: 51 (99); n = 800: 76
+    //    (132); B = 32, n = 1000, degree 64: 37 (61)); below the line it would win too
+    //    at n = 1200 and 1400, degree 64 (B = 128: 142 (293) and 173 (300));
+    //  * with few tiles from 32 + n / 20 up, by 14 / tiles higher below 100 tiles, and
+    //    not below 24 (ticks, one graph: n = 1000, degree 100, B = 32 1.56 of the
+    //    staged kernel's time, B = 128 1.02; n = 850, 4 graphs, degree 110 1.20, 160 1.08);
+    //  * MaxCut meets x inside the box for longer, whose rows it sums in CSR order:
+    //    against the shared-memory kernel from 48 + n / 16 (64 graphs, B = 32: n = 600,
+    //    degree 96: 38.5 (57); ticks 0.8 and late ones 0.6 of the other's time; plain
+    //    steps from x all over the box 1.05 to 1.4), not for the smallest graphs at
+    //    B = 32 (n = 160: 1.2); else from 16 + n / 25 (B = 128, n = 800, degree 48: 114
+    //    (146), n = 1000, degree 64: 189 (181), n = 1700, degree 96: 392 (480); float16
+    //    676 (505)), with few tiles as below (ticks, one graph, B = 32: n = 1000, degree
+    //    200 2.3 of the staged kernel's time, B = 128, n = 800, degree 110 1.5, 160 0.95).
     s->dense_ok = g->d_bits != nullptr && p->x_dtype != DT_F32 && B % kDenseGroup == 0;
     if (s->dense_ok) {
       s->dense_plan.bits = g->d_bits;
@@ -1070,16 +1085,20 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
       const int pairs = (dense_tiles(g->max_ng) + 1) / 2;
       const int ctas = g->G * (B / kDenseGroup);
       s->dense_plan.parts = std::max(1, std::min(pairs, (6 * g->sms + ctas - 1) / ctas));
-      const double degree = (double)g->nnz / (double)g->n;
-      const bool fills = (int64_t)ctas * dense_tiles(g->max_ng) >= g->sms;
-      // MaxCut meets x inside the box for longer (rows summed in CSR order), and
-      // 11-bit significands leave fewer sums exact: a higher line against the
-      // shared-memory kernel, and none for float16 (407 graphs, n = 164, degree
-      // 46, B = 128: 164 us a tick against 142)
+      const double degree = (double)g->nnz / (double)g->n, n = g->max_ng;
+      const int64_t tiles = (int64_t)ctas * dense_tiles(g->max_ng);
+      const bool fills = tiles >= g->sms, smem = s->step_smem_max > 0;
+      // 11-bit significands leave fewer sums exact: MaxCut in float16 stays with the
+      // shared-memory kernel (407 graphs, n = 164, degree 46, B = 128: 164 us a tick
+      // against 142)
       const bool cut = p->problem == PROB_MAXCUT;
-      const double from = s->step_smem_max > 0 || !fills ? (cut ? 48.0 + g->max_ng / 16.0 : 32.0 + g->max_ng / 20.0)
-                                                         : 16.0 + g->max_ng / 25.0;
-      const bool few_exact = cut && p->x_dtype == DT_F16 && s->step_smem_max > 0;
+      double from;
+      if (smem && cut) from = n <= 256 && B == 32 ? 1e9 : 48.0 + n / 16.0;
+      else if (smem) from = fills ? 32.0 + n / 20.0 : 38.0 + n / 18.0;
+      else if (fills) from = 16.0 + n / 25.0;
+      else if (cut) from = tiles < 28 ? 1e9 : std::max(48.0 + n / 16.0, tiles < 76 ? 0.18 * n : 0.0);
+      else from = tiles < 24 ? 1e9 : (32.0 + n / 20.0) * (tiles < 100 ? 1.0 + 14.0 / (double)tiles : 1.0);
+      const bool few_exact = cut && p->x_dtype == DT_F16 && smem;
       if ((!force && !ellv && !c16 && degree >= from && !few_exact) || (force && strcmp(force, "dense") == 0))
         s->dense = &s->dense_plan;
     }

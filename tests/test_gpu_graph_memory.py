@@ -21,7 +21,7 @@ if os.environ.get("FAIL"):
 g = mq.Graph(P)
 os.environ.pop("SHIM_FAIL_BYTES", None)
 s = mq.Solver(g, mq.params(batch=32, x_dtype=1, t_gs=2, descent_cap=20, seed=3))
-assert s.info()["dense"] == (not os.environ.get("FAIL")), s.info()
+assert s.info()["disc_bits"] == (not os.environ.get("FAIL")), s.info()
 s.run(60)
 s.local_search()
 v, bits = s.best()
