@@ -1175,10 +1175,11 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
         const double degree = (double)g->nnz / (double)g->n, load = (double)items / g->sms;
         const bool f32 = p->x_dtype == DT_F32;
         const bool mis = p->problem == PROB_MIS;
-        const double least = items <= 32 ? (!mis || B == 128 ? 0.0 : B == 64 ? 20e3 : 28e3)
+        const double least = items <= 32 || B < 32 ? (!mis || (B != 32 && B != 64) ? 0.0 : B == 64 ? 20e3 : 28e3)
                                          : (B == 32 ? (mis ? 50e3 : 30e3) : B == 64 ? 28e3 : f32 ? 0.0 : 31e3);
         const double gathered = (double)g->nnz * B / items;
-        const bool long_rows = f32 && (B < 128 ? items * degree > 900.0 : items * degree > 1300.0 && gathered < 300e3);
+        const bool long_rows = f32 && B >= 32 && items > 32 &&
+                               (B < 128 ? items * degree > 900.0 : items * degree > 1300.0 && gathered < 300e3);
         const bool few = 3 * items < g->sms && (s->staged_ok || rows) && gathered >= least && !long_rows;
         const double most = load < 0.5    ? (B == 32 ? 48.0 : 1e9)
                             : load < 0.75 ? (B == 32 ? 32.0 : B == 64 ? 48.0 : 1e9)
