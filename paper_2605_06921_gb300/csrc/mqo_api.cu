@@ -714,6 +714,13 @@ mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
   return es;
 }
 
+// Discrete rounds follow one another: descents are cut off after a few steps
+// (MIS repairs each), or few of them lie between two local searches.
+bool rounds_often(const mqo_params& p) {
+  return (p.problem == PROB_MIS && p.repair && p.descent_cap < 20) ||
+         (p.local_search && ((int64_t)p.t_gs + 1) * p.descent_cap < 300);
+}
+
 // Is a tick of the machine in the multi-tick kernel no slower than one of the
 // tick's kernels?  Ticks with discrete rounds cost it more than steps do (a
 // CTA walks all lists of its member graph), so where descents are short, so that
@@ -729,8 +736,7 @@ mqo_solver_s::EllSet ell_set(mqo_solver s, bool wide) {
 bool tick_small_faster(mqo_solver s, const mqo_params& p, int pairs, int64_t work, int waves) {
   const mqo_graph g = s->g;
   const bool mis = p.problem == PROB_MIS, bits = g->d_bits != nullptr && p.batch >= 32;
-  const bool rounds = (mis && p.repair && p.descent_cap < 20) ||
-                      (p.local_search && ((int64_t)p.t_gs + 1) * p.descent_cap < 300);
+  const bool rounds = rounds_often(p);
   if (!mis && !rounds) return true;
   struct Cost {
     double base, pair, work, node;                        // multi-tick kernel
@@ -1222,10 +1228,21 @@ mqo_status mqo_solver_create(mqo_graph g, const mqo_params* p, void* cuda_stream
     s->disc_smem_max = (B >= 32 && dneed <= kDiscSmemLimit && (!few || fused)) ? dneed : 0;
     s->disc_smem = pairs ? 0 : s->disc_smem_max;
     // Member graphs with bit matrices: the form that follows the trajectories in
-    // a round (MQO_DISC_KERNEL=bits where possible; the others exclude it).
+    // a round (MQO_DISC_KERNEL=bits where possible; the others exclude it).  Where
+    // rounds follow one another most trajectories are in one, which the lists serve
+    // a word at a time.  Measured (us of a tick, descents of 6 steps, bits against
+    // the fused lists): MIS, 152 graphs, B = 64: n = 100, degree 10 66 and 41, degree 30
+    // 56 and 40, n = 200, degree 36 78 and 63, degree 80 1.0 of the other's time, n = 400,
+    // degree 30 up to 1.3, MaxCut 0.3 to 1.2 of it; against the node-parallel lists:
+    // one graph, B = 32: n = 800, degree 120 60 and 48, MaxCut 102 and 45, n = 1200,
+    // degree 200 104 and 64, 178 and 59; n = 400 and below 0.2 to 1.3 of it.
+    const double degree = (double)g->nnz / (double)g->n;
+    const bool mis = p->problem == PROB_MIS;
+    const bool lists = rounds_often(*p) && (few ? max_ng >= 700 && g->G <= 16 && (B == 32 || (B == 64 && !mis && degree >= 100.0))
+                                                : mis && s->disc_smem_max > 0 && degree < 48.0);
     s->disc_bits_max = g->d_bits != nullptr && B >= 32 ? disc_bits_smem_bytes(p->problem, max_ng) : 0;
     if (s->disc_bits_max > kDiscBitsSmemLimit) s->disc_bits_max = 0;
-    if (s->disc_bits_max > 0 && (!dforce || strcmp(dforce, "bits") == 0)) {
+    if (s->disc_bits_max > 0 && (dforce ? strcmp(dforce, "bits") == 0 : !lists)) {
       s->disc_bits = true;
       s->disc_smem = s->disc_bits_max;
     }
