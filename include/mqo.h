@@ -319,7 +319,8 @@ MQO_API mqo_status mqo_traj_state(mqo_solver s, mqo_traj_info* out);
  * they fit, bit 19 set or not), bit 20 = the row-group kernel (16-bit x,
  * neighbour rows read from L2, bits 0 and 3 clear), bit 21 = the fused
  * discrete passes run on the bit matrices of dense member graphs (bit 1 is set
- * too); *smem_bytes = the
+ * too), bit 22 = a tick's discrete passes follow its step (they run beside it
+ * otherwise); *smem_bytes = the
  * shared-memory step kernel's dynamic shared memory per CTA; *items = work
  * items (node ranges of at most 256 nodes); *replicas = counter replicas per
  * trajectory.

@@ -52,7 +52,8 @@ def _plan(p):
         kern = "staged" if p & 8 else "rows" if p & (1 << 20) else "global"
     return {"step_kernel": kern, "discrete_kernel": "graph" if p & 2 else "pairs", "lanes_vec": (p >> 4) & 15,
             "slice_kb": (p >> 8) & 255, "col16": bool(p & (1 << 16)), "ell": bool(p & (1 << 17)),
-            "dense": bool(p & (1 << 18)), "small": bool(p & (1 << 19)), "disc_bits": bool(p & (1 << 21))}
+            "dense": bool(p & (1 << 18)), "small": bool(p & (1 << 19)), "disc_bits": bool(p & (1 << 21)),
+            "step_first": bool(p & (1 << 22))}
 
 
 class TrajInfo(C.Structure):
@@ -290,8 +291,8 @@ class Solver:
 
     def info(self):
         """Execution plan: step kernel (smem, smem_wide, staged, rows or global; dense: the tensor-core kernel instead),
-        small (many ticks per launch), discrete kernel (disc_bits: on bit matrices), trajectories per lane, KB of gathered
-        rows per staged slice, smem bytes, items, counter replicas."""
+        small (many ticks per launch), discrete kernel (disc_bits: on bit matrices; step_first: after the step, not beside it),
+        trajectories per lane, KB of gathered rows per staged slice, smem bytes, items, counter replicas."""
         k, sm, it, r = C.c_int32(), C.c_int64(), C.c_int32(), C.c_int32()
         _check(lib().mqo_solver_info(self.handle, C.byref(k), C.byref(sm), C.byref(it), C.byref(r)))
         return dict(_plan(k.value), smem_bytes=sm.value, items=it.value, replicas=r.value)

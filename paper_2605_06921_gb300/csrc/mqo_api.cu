@@ -778,6 +778,26 @@ bool serial_tick() {
   return e && strcmp(e, "1") == 0;
 }
 
+// Do the plan's step and fused discrete kernel run one after the other?  A
+// shared-memory step of one wave (a CTA on each SM) that starts beside the
+// discrete kernel's CTAs finds their SMs taken and puts two of its own on
+// others, which halves the step's speed where gathers bound it (16-byte lanes,
+// float32); with rare rounds the discrete CTAs end at once and nothing is
+// gained by the overlap.  Measured (us of a tick, beside and after; rounds
+// rare, bit matrices): MaxCut, 75 graphs, n = 300, degree 60, float16: B = 64
+// 71.2 and 47.5, B = 128 129.9 and 82.0; MIS, 76 graphs, n = 200, degree 36, B = 128
+// 51.1 and 40.7; float32, 100 graphs, n = 120, degree 40, B = 128 65.7 and 43.8.
+// 8-byte lanes 0.98 to 1.04, more items than SMs 0.94 to 1.06, rounds often
+// 1.05 to 1.4: beside.
+bool one_wave(mqo_solver s) {
+  const mqo_graph g = s->g;
+  const SolverDev& S = s->S;
+  if (s->disc_smem == 0 || s->step_smem == 0 || s->dense || rounds_often(s->p)) return false;
+  if (!S.step_wide && S.p.x_dtype != DT_F32) return false;
+  const int disc = s->disc_bits ? disc_bits_ctas(S, g->sms) : g->G;
+  return g->num_items <= g->sms && g->num_items + disc > g->sms;
+}
+
 // the discrete passes fused into one launch
 cudaError_t launch_disc_fused(mqo_solver s, cudaStream_t stream) {
   if (s->disc_bits) return launch_disc_bits(s->S, s->g->d_bits, s->g->d_bits_off, s->disc_smem, s->g->sms, stream);
@@ -794,7 +814,7 @@ cudaError_t enqueue_tick(mqo_solver s) {
   }
   if ((e = launch_ctrl(S, CTRL_MACHINE, nullptr, s->work)) != cudaSuccess) return e;
   if ((e = launch_apply(S, s->work)) != cudaSuccess) return e;
-  if (s->work2 && !serial_tick()) {
+  if (s->work2 && !serial_tick() && !one_wave(s)) {
     // The step (x, V, rounding words; counters of stepping trajectories) and
     // the discrete passes (work, auxiliary, free and drop bit sets and the
     // move arrays; counters of trajectories in a round, integer atomics)
@@ -1572,7 +1592,8 @@ mqo_status mqo_solver_info(mqo_solver s, int32_t* step_kernel, int64_t* smem_byt
                    ((staged ? slice_kb(s) : 0) << 8) |
                    ((s->step_smem > 0 && s->S.step_c16 && !s->dense) ? (1 << 16) : 0) |
                    ((s->step_smem > 0 && s->step_ell && !s->dense) ? (1 << 17) : 0) | (s->dense ? (1 << 18) : 0) |
-                   (s->small ? (1 << 19) : 0) | (rows ? (1 << 20) : 0) | (s->disc_bits ? (1 << 21) : 0);
+                   (s->small ? (1 << 19) : 0) | (rows ? (1 << 20) : 0) | (s->disc_bits ? (1 << 21) : 0) |
+                   (one_wave(s) ? (1 << 22) : 0);
   if (smem_bytes) *smem_bytes = (int64_t)(s->dense ? s->dense->smem : s->step_smem);
   if (items) *items = s->S.g.num_items;
   if (replicas) *replicas = s->S.R;
@@ -1999,7 +2020,7 @@ mqo_status mqo_autotune(mqo_solver s, int32_t ticks, int32_t* plan_out, double* 
                 (stg ? 8 : 0) | (chosen.vec << 4) | ((stg ? chosen.slice_kb : 0) << 8) |
                 ((chosen.step_smem > 0 && chosen.c16) ? (1 << 16) : 0) |
                 ((chosen.step_smem > 0 && chosen.ell) ? (1 << 17) : 0) | (rows ? (1 << 20) : 0) |
-                (chosen.dbits ? (1 << 21) : 0);
+                (chosen.dbits ? (1 << 21) : 0) | (one_wave(s) ? (1 << 22) : 0);
   }
   if (best_ms_per_tick) *best_ms_per_tick = best / ticks;
   return MQO_OK;

@@ -495,17 +495,21 @@ size_t disc_bits_smem_bytes(int problem, int max_ng) {
   return n * (3 * 4 + kDbBatch * (4 + 4 + 2 + (problem == PROB_MIS ? 0 : 4))) + 16;
 }
 
-cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, size_t smem,
-                             int sms, cudaStream_t stream) {
-  // a CTA per member graph and word of trajectories while there are SMs for
-  // them, else a CTA takes several words (one CTA fits on an SM, and a tick
-  // without rounds pays for the launch of each: 407 graphs, B = 128: 9.8 us with
-  // a CTA per word, 7.3 with one per graph)
+// a CTA per member graph and word of trajectories while there are SMs for
+// them, else a CTA takes several words (one CTA fits on an SM, and a tick
+// without rounds pays for the launch of each: 407 graphs, B = 128: 9.8 us with
+// a CTA per word, 7.3 with one per graph)
+int disc_bits_ctas(const SolverDev& S, int sms) {
   int parts = S.Bw;
   while (parts > 1 && S.g.num_graphs * parts > sms) parts /= 2;
+  return S.g.num_graphs * parts;
+}
+
+cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, size_t smem,
+                             int sms, cudaStream_t stream) {
   cudaError_t e = allow_smem(k_disc_bits, kDiscBitsSmemLimit);
   if (e != cudaSuccess) return e;
-  k_disc_bits<<<S.g.num_graphs * parts, kDbThreads, smem, stream>>>(S, bits, bits_off);
+  k_disc_bits<<<disc_bits_ctas(S, sms), kDbThreads, smem, stream>>>(S, bits, bits_off);
   return cudaGetLastError();
 }
 

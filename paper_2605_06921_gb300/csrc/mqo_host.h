@@ -78,6 +78,7 @@ size_t disc_graph_smem_bytes(int B, int max_ng);
 cudaError_t launch_disc_graph(const SolverDev& S, size_t smem, cudaStream_t stream);
 // the same for member graphs with bit matrices (mqo_disc_bits.cu)
 size_t disc_bits_smem_bytes(int problem, int max_ng);
+int disc_bits_ctas(const SolverDev& S, int sms);
 cudaError_t launch_disc_bits(const SolverDev& S, const uint4* bits, const int64_t* bits_off, size_t smem,
                              int sms, cudaStream_t stream);
 cudaError_t launch_tick_end(const SolverDev& S, cudaStream_t stream);
