@@ -417,6 +417,13 @@ STEP_SOURCES = {"smem": ("mqo_step.cu", "mqo_step_smem.cuh", "mqo_step.cuh", "mq
                 "f32_ell": ("mqo_step_f32.cu", "mqo_step.cuh", "mqo_dev.cuh")}
 
 
+def float32_stream(plan, x_dtype, batch=32):
+    """Does the plan's step stage its member graphs' x as float32 (16-bit
+    offsets in the sliced-ELL stream)?  Float32 states and fewer than 32
+    trajectories of any type do where they take the stream."""
+    return bool(plan.get("ell")) and (x_dtype == "f32" or batch < 32)
+
+
 def step_variant(plan):
     """Profile variant name of a plan: smem, smem_wide (CSR indices),
     smem_ell, smem_wide_ell (sliced-ELL stream), staged, rows, global, dense
@@ -427,9 +434,9 @@ def step_variant(plan):
     return kern + "_ell" if kern.startswith("smem") and plan.get("ell") else kern
 
 
-def step_kernel_traffic(workload, x_dtype, variant):
+def step_kernel_traffic(workload, x_dtype, variant, batch=32):
     """DRAM bytes per launch of the step kernel variant (step_variant)."""
-    if x_dtype == "f32" and variant == "smem_wide_ell":
+    if float32_stream({"ell": variant == "smem_wide_ell"}, x_dtype, batch):
         variant = "f32_ell"
     if variant in STEP_SOURCES and not variant.startswith("smem"):
         src = STEP_SOURCES[variant]
@@ -597,13 +604,13 @@ STEP_KERNEL_NAMES = {"smem": "mqo::k_step_s", "smem_wide": "mqo::k_step_s", "sta
                      "global": "mqo::k_step_g", "rows": "mqo::k_step_r"}
 
 
-def step_kernel_name(plan, x_dtype):
+def step_kernel_name(plan, x_dtype, batch=32):
     """The kernel that runs a plan's steps."""
     if plan.get("small"):
         return "mqo::k_small (many ticks per launch)"
     if plan.get("dense"):
         return "mqo::k_step_t"
-    if x_dtype == "f32" and plan.get("ell"):
+    if float32_stream(plan, x_dtype, batch):
         return "mqo::k_step_f"
     return STEP_KERNEL_NAMES.get(plan["step_kernel"], plan["step_kernel"])
 
@@ -627,8 +634,9 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
     read and written once, rounding words) per launch over its average
     launch time; the shared-memory kernel adds its gather bound."""
     # index bytes per CSR entry: 16-bit member-local ids, 32-bit ids, or the
-    # sliced-ELL stream's row offsets (its padding not counted; float32 x: 16 bits)
-    idx = (2 if x_dtype == "f32" else 4) if plan.get("ell") else (2 if plan.get("col16") else 4)
+    # sliced-ELL stream's row offsets (its padding not counted; x staged as float32: 16 bits)
+    f32_stream = float32_stream(plan, x_dtype, B)
+    idx = (2 if f32_stream else 4) if plan.get("ell") else (2 if plan.get("col16") else 4)
     alg = algorithmic_bytes_per_step(G, B, sx, sv, idx)
     if plan.get("dense"):  # bit matrices (rows and columns padded to 128) in place of the column indices
         rows = -(-member_sizes(G) // 128) * 128
@@ -637,8 +645,8 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
     hbm = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
            "algorithmic_bytes_per_launch": alg, "peak_source": peak_src}
     kern = plan["step_kernel"]
-    traffic = step_kernel_traffic(workload, x_dtype, step_variant(plan))
-    gathered = float(G.nnz) * B * sx  # neighbour rows of x read per launch
+    traffic = step_kernel_traffic(workload, x_dtype, step_variant(plan), B)
+    gathered = float(G.nnz) * B * (4 if f32_stream else sx)  # neighbour rows of x read per launch
     if plan.get("dense"):
         # the adjacency comes from bit matrices and x once per CTA
         flops = dense_flops_per_step(G, B)
@@ -664,7 +672,7 @@ def step_roofline(G, B, sx, sv, step_ms, plan, workload, x_dtype, hbm_peak, peak
         # is DRAM traffic on top of the algorithmic bytes (measured: traffic)
         roof = dict(hbm, traffic=traffic, gathered_bytes_per_launch=gathered,
                     achieved_incl_gathers=(alg + gathered) / (step_ms / 1e3) / 1e9)
-    roof.update(kernel=step_kernel_name(plan, x_dtype), step_kernel_ms=step_ms, plan=plan)
+    roof.update(kernel=step_kernel_name(plan, x_dtype, B), step_kernel_ms=step_ms, plan=plan)
     if traffic:
         # DRAM bytes of the committed capture over this launch time, against the same peak
         roof["dram_gbs_from_traffic"] = traffic / (step_ms / 1e3) / 1e9
