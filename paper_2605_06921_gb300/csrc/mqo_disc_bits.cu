@@ -14,7 +14,8 @@
 // a row is read once for kDbBatch trajectories.  Bound by the latency of the
 // rows' words (L2) and of the block barriers.
 //
-// One CTA per (member graph, word of 32 trajectories).
+// One CTA per (member graph, word of 32 trajectories), or a CTA takes several
+// words of its graph where the graphs are many (disc_bits_ctas).
 #include "mqo_dev.cuh"
 #include "mqo_host.h"
 
@@ -159,14 +160,12 @@ __global__ void __launch_bounds__(kDbThreads) k_disc_bits(SolverDev S, const uin
       // ---------------- pass A: decisions on the snapshot
       uint32_t change[(2048 + kDbThreads - 1) / kDbThreads];  // per own row: bit k = this row's bit changes
       if (rounds) {
-        int i = 0;
 #pragma unroll
         for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) change[q] = 0u;
 #pragma unroll
         for (int q = 0; q < (2048 + kDbThreads - 1) / kDbThreads; ++q) {
           const int v = threadIdx.x + q * kDbThreads;
           if (v >= n) break;
-          ++i;
           const int wv = v >> 5;
           const uint32_t pb = 1u << perm(v & 31), lt = below(v & 31);
           bool some[kDbBatch];  // some smaller neighbour in the round's set
