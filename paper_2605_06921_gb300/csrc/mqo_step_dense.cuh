@@ -22,12 +22,12 @@
 // one by one in CSR order; a warp with many of them sums its 32 rows again,
 // and a block of x with many small values skips the product.
 //
-// Measured (BF16, one step): 512 graphs, n ~ 750, degree 112, B = 32: 162 us
-// (sliced ELL) -> 86 us, 97 us inside the machine; 8 graphs (1000, 100), B = 128:
+// Measured (BF16, one step): 512 graphs, n ~ 750, degree 112, B = 32, inside the
+// machine: 162 us (sliced ELL) -> 104 us; 8 graphs (1000, 100), B = 128:
 // 130 (staged) -> 24 us; 8 graphs (1000, 500), B = 128, MaxCut: 264 -> 27 us on
 // binary points, 150 us with every row summed in CSR order.  Bound by the
-// latency between the warps that expand A and the MMAs (tensor pipe 30 %
-// active, issue about half): TMEM holds two chunks of A per row tile.
+// latency between the warps that expand A and the MMAs (tensor pipe 20 %
+// active, issue 42 %): TMEM holds two chunks of A per row tile.
 #pragma once
 
 #include "mqo_step.cuh"
